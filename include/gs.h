@@ -139,6 +139,10 @@ typedef struct {
  *     (V - k) x (200 B per Gaussian + 16 B per instance of a view) plus the
  *     loss maps; k = 4 keeps the projection reading each Gaussian once per
  *     4 views, as in a plan without recompute.
+ * Tiles of whole 8x8 pixel blocks (8x8, 16x8, 16x16, 32x8, ...) are rendered by
+ * kernels that give a warp a block whatever the batch sizes and pixels per
+ * thread say; these are checked all the same, and shape the launches of the
+ * other tiles and of deterministic plans of larger tiles.
  * The tile shape changes which pixels a Gaussian can reach (its 3-sigma
  * rect is counted in whole tiles), hence the image; the batch sizes, pixels
  * per thread, tight_rect and recompute change only the speed and memory. */

@@ -1,0 +1,901 @@
+// gs_blocks.cu -- A5 forward compositing and A7 pixel adjoint over 8x8 pixel
+// blocks, for tiles that are whole 8x8 blocks.
+//
+// A warp owns one 8x8 block of a tile: lane l holds the two pixels of row l / 4
+// at columns 2 (l % 4) and the next one.  It walks its tile's list on its own,
+// so nothing in these kernels waits for another warp.
+//
+//  * Staging.  32 list entries at a time, one per lane: the lane's record
+//    arrives by cp.async, is turned into tile-local coordinates and, where the
+//    tile is more than the block or its list is a square rect's, tested
+//    against the block (the smallest value of the Gaussian's quadratic form
+//    over the block's rectangle).  The Gaussians that can reach the block are
+//    packed into the warp's stage two by two: {x, x', y, y'}, {-a/2, -a'/2, -b, -b'},
+//    {-c/2, -c'/2, -o, -o'}, so that one packed FP32 operation (.f32x2) evaluates
+//    both at a pixel with no register shuffled into pairs.
+//  * The forward blends front to back, the adjoint walks back to front; both
+//    evaluate alpha with the same rounded operations as gs_render.cu and take
+//    the same decisions.
+//  * The adjoint's sums over the block.  Per blended Gaussian the 64 pixels'
+//    dL/dpower and blend weights go to shared memory as one row of a window;
+//    eight rows make the A operand of mma.sync m16n8k8 (TF32 inputs, FP32
+//    sums), with each value split into two TF32 parts (rows 0-7 the high
+//    parts, rows 8-15 the low ones), against the monomials 1, x, y, x^2, xy,
+//    y^2 of the pixel's place in the block (exact in TF32) and against dL/dC
+//    (split the same way).  The moments about the Gaussian's mean follow from
+//    those about the block's centre.
+//
+// What bounds them: instruction issue and the ALU and heavy FMA pipes, two
+// cycles per instruction each (packed FP32 runs on the heavy pipe alone), and
+// for small launches the longest list, which one warp walks.  At 1M Gaussians,
+// 1200x680, 8x8 tiles (2.0M walked (block, Gaussian) pairs), against the kernels
+// of gs_render.cu at their best launch shape: forward 179 -> 137 us, 85 -> 51
+// warp instructions per pair; adjoint 330 -> 265 us, 138 -> 97 (the sums over the
+// block by shuffles took 43 of them, the window takes 24).  Sixteen views of a
+// 500k map: 1003 -> 645 and 1593 -> 1451 us.  200k Gaussians, 640x480, 16x16
+// tiles: 68 -> 45 and 177 -> 85 us (there the block test and the four warps per
+// tile count as well).  Tried in the adjoint and not kept: the high parts
+// rounded instead of cut (1503 us), a Newton step on 1 / (1 - alpha) (1476 us):
+// neither moved the gradients' error against 64 bits.
+#include "gs_render.cuh"
+
+namespace gs {
+namespace {
+
+constexpr int kBlock = 8;      // pixels along each side of a block
+constexpr int kWarps = 4;      // warps (blocks) per CTA
+constexpr int kChunk = 32;     // list entries staged at a time, one per lane
+constexpr unsigned kAll = 0xffffffffu;
+
+// e^p = 2^(p log2 e) by the hardware's base-2 exponential (ex2.approx.ftz): the
+// results below 2^-126 that it flushes to zero are far below 1/255.
+constexpr float kLog2e = 1.4426950408889634f;
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+
+// A warp's staged Gaussians.  par: pairs of slots; col: the colour, each
+// channel twice, and the slot's tag (the list position in the forward, the
+// list value in the adjoint).
+template <int SLOTS>
+struct Stage {
+    float4 par[SLOTS / 2][3];
+    float4 col[SLOTS][2];
+};
+
+// Whether the Gaussian's alpha can reach 1/255 in the pixels [x0, x0 + 7] x
+// [y0, y0 + 7]: q(d) = a dx^2 + 2 b dx dy + c dy^2 against 2 ln(255 o), the
+// level widened by 1% + 0.02, far beyond the rounding of either side.  The
+// smallest q over a rectangle that does not hold the mean lies on one of the
+// two edges that face it.
+__device__ __forceinline__ bool meets_block(float lx, float ly, float a, float b, float c,
+                                            float o, float x0, float y0) {
+    const float xe = fminf(fmaxf(lx, x0), x0 + 7.0f) - lx;
+    const float ye = fminf(fmaxf(ly, y0), y0 + 7.0f) - ly;
+    const float dy = fminf(fmaxf(__fdividef(-b * xe, c), y0 - ly), y0 + 7.0f - ly);
+    const float dx = fminf(fmaxf(__fdividef(-b * ye, a), x0 - lx), x0 + 7.0f - lx);
+    const float q1 = fmaf(a * xe, xe, fmaf(2.0f * b * xe, dy, c * dy * dy));
+    const float q2 = fmaf(a * dx, dx, fmaf(2.0f * b * dx, ye, c * ye * ye));
+    const float level = 2.02f * __logf(255.0f * o) + 0.02f;
+    return !(fminf(q1, q2) > level);
+}
+
+// One chunk of a list on its way through a warp's raw buffer into its stage.
+// RING chunks are in flight.
+template <int SLOTS, int RING>
+struct Feeder {
+    float4* raw;  // RING x kChunk x 3
+    Stage<SLOTS>* st;
+    const uint32_t* __restrict__ ivals;
+    const uint32_t* __restrict__ gid_of;
+    const float4* __restrict__ rec;
+    uint32_t next;         // this lane's list value of the next chunk to issue
+    uint32_t tag[RING];    // ... and of the chunks in flight
+    int issued;            // chunks issued so far
+    bool odd;              // some colour of the batch is not finite (forward)
+
+    // pos(c): this lane's position in the list in chunk c, or -1
+    template <class Pos>
+    __device__ __forceinline__ void load_next(const Pos& pos) {
+        const int p = pos(issued);
+        next = p >= 0 ? __ldg(ivals + p) : 0u;
+    }
+    template <class Pos>
+    __device__ __forceinline__ void issue(const Pos& pos, int slot, int lane) {
+        const int p = pos(issued);
+        tag[slot] = next;
+        if (p >= 0) {
+            const uint32_t vg = gid_of ? __ldg(gid_of + next) : next;
+            const float4* src = rec + (size_t)vg * 3;
+            float4* dst = raw + (slot * kChunk + lane) * 3;
+            cp_async16(dst, src);
+            cp_async16(dst + 1, src + 1);
+            cp_async16(dst + 2, src + 2);
+        }
+        cp_async_commit();
+        ++issued;
+        load_next(pos);
+    }
+    template <class Pos>
+    __device__ __forceinline__ void start(const Pos& pos, int lane) {
+        issued = 0;
+        load_next(pos);
+#pragma unroll
+        for (int i = 0; i < RING; ++i) issue(pos, i, lane);
+    }
+    // Stages chunk c behind the ns slots in use; returns the lanes whose entry
+    // was kept.  LISTPOS: the tag is the list position instead of the value.
+    template <int CH, bool CULL, bool LISTPOS, class Pos>
+    __device__ __forceinline__ unsigned stage(const Pos& pos, int c, int ns, int lane, float tx0,
+                                              float ty0, float bx, float by, int list_base) {
+        if (RING == 1) cp_async_wait_all(); else cp_async_wait_one();
+        __syncwarp();
+        const int slot = RING == 1 ? 0 : (c & (RING - 1));
+        const int p = pos(c);
+        float4 m, q, col = make_float4(0.f, 0.f, 0.f, 0.f);
+        bool keep = p >= 0;
+        if (keep) {
+            const float4* src = raw + (slot * kChunk + lane) * 3;
+            m = src[0];
+            q = src[1];
+            col = src[2];
+            m.x = __fadd_rn(__fsub_rn(m.x, tx0), m.z);
+            m.y = __fadd_rn(__fsub_rn(m.y, ty0), m.w);
+            if (CULL) keep = meets_block(m.x, m.y, q.x, q.y, q.z, q.w, bx, by);
+        }
+        const uint32_t t = RING == 1 || slot == 0 ? tag[0] : tag[RING - 1];
+        const unsigned mask = __ballot_sync(kAll, keep);
+        if (LISTPOS) {
+            const bool fin = fabsf(col.x) < INFINITY && fabsf(col.y) < INFINITY &&
+                             fabsf(col.z) < INFINITY;
+            odd = (ns > 0 && odd) || __any_sync(kAll, keep && !fin);
+        }
+        if (RING == 1 || slot == 0) issue(pos, 0, lane); else issue(pos, RING - 1, lane);
+        if (keep) {
+            const int s = ns + __popc(mask & ((1u << lane) - 1u));
+            float* f = reinterpret_cast<float*>(&st->par[s >> 1][0]) + (s & 1);
+            f[0] = m.x;
+            f[2] = m.y;
+            f[4] = -0.5f * q.x;
+            f[6] = -q.y;
+            f[8] = -0.5f * q.z;
+            f[10] = -q.w;
+            const float word = __uint_as_float(LISTPOS ? (uint32_t)(p - list_base) : t);
+            if (CH == 3) {
+                st->col[s][0] = make_float4(col.x, col.x, col.y, col.y);
+                st->col[s][1] = make_float4(col.z, col.z, word, 0.0f);
+            } else {
+                const float g = (col.x + col.y + col.z) * (1.0f / 3.0f);
+                st->col[s][0] = make_float4(g, g, word, 0.0f);
+            }
+        }
+        return mask;
+    }
+    // A last pair with one slot in use: the other half never reaches a pixel.
+    __device__ __forceinline__ void pad(int ns, int lane) {
+        if (!(ns & 1)) return;
+        if (lane < 6) reinterpret_cast<float*>(&st->par[ns >> 1][0])[2 * lane + 1] = 0.0f;
+        if (lane < 8) reinterpret_cast<float*>(&st->col[ns][0])[lane] = 0.0f;
+    }
+    // Whether a staged Gaussian may need what most do not: it can reach alpha =
+    // 0.99 (o >= 0.99), or its conic is so close to singular that rounding could
+    // make its power positive.  With b^2 <= (1 - e) a c the exact power is at
+    // most -e/4 (a dx^2 + c dy^2) and its rounding error below 4e-7 times the
+    // same sum: e = 1e-5.
+    __device__ __forceinline__ bool hard(int ns, int lane) const {
+        bool h = false;
+#pragma unroll
+        for (int k = 0; k < SLOTS / 64; ++k) {
+            const int p = lane + 32 * k;
+            if (2 * p < ns) {
+                const float4 B = st->par[p][1], D = st->par[p][2];
+                h = h || !(D.z > -kAlphaMax && D.w > -kAlphaMax &&
+                           B.z * B.z <= 3.99996f * B.x * D.x &&
+                           B.w * B.w <= 3.99996f * B.y * D.y);
+            }
+        }
+        return __any_sync(kAll, h);
+    }
+};
+
+// -o e^power of two Gaussians (the halves) at one pixel, and their powers.
+struct PairAlpha {
+    float2 pw, noG;
+};
+// hcdd, ha: -c dy^2 / 2 and -a / 2 (halving is exact, so the power -(a dx^2 + c
+// dy^2) / 2 - b dx dy is rounded as gauss_power rounds it).
+__device__ __forceinline__ PairAlpha pair_alpha(float2 dx, float2 dy, float2 hcdd, float2 ha,
+                                                float2 nb, float2 no) {
+    PairAlpha r;
+    const float2 q = fma2(ha, mul2(dx, dx), hcdd), t = mul2(nb, mul2(dx, dy));
+    // (scalar sums: a packed product whose only use is a packed sum is fused
+    // with it, which rounds once instead of twice)
+    r.pw = make_float2(__fadd_rn(q.x, t.x), __fadd_rn(q.y, t.y));
+    r.noG = mul2(no, make_float2(ex2_approx(r.pw.x * kLog2e), ex2_approx(r.pw.y * kLog2e)));
+    return r;
+}
+// ... with alpha clamped at 0.99 and no weight at a positive power, for the
+// pairs that hard_pairs names (the others reach neither).
+__device__ __forceinline__ float2 tame(const PairAlpha& e) {
+    return make_float2(e.pw.x <= 0.0f ? fmaxf(-kAlphaMax, e.noG.x) : 0.0f,
+                       e.pw.y <= 0.0f ? fmaxf(-kAlphaMax, e.noG.y) : 0.0f);
+}
+
+// ---------------------------------------------------------------------------
+// Forward.
+// ---------------------------------------------------------------------------
+
+template <int CH>
+struct FwdPixels {
+    float2 T, C[CH];  // transmittance, negated once the pixel is done; minus the colour
+    int l0, l1;       // slot of the last blended Gaussian of this batch, or -1
+};
+
+// Blends one Gaussian (n = -alpha where it counts at the pixel, else 0) at both
+// pixels without a branch: alpha zero leaves a pixel as it is; the Gaussian
+// that would take T below 1e-4 is not added and negates T, after which nothing
+// passes the test of Tn.
+template <int CH>
+__device__ __forceinline__ void blend_one(FwdPixels<CH>& s, float2 na, const float4* col,
+                                          int slot) {
+    const float2 Tn = mul2(s.T, make_float2(1.0f + na.x, 1.0f + na.y));
+    const bool a0 = Tn.x >= kTMin, a1 = Tn.y >= kTMin;
+    const float2 w = mul2(na, s.T);
+    const float2 nw = make_float2(a0 ? w.x : 0.0f, a1 ? w.y : 0.0f);
+    const float4 c01 = col[0];
+    s.C[0] = fma2(nw, make_float2(c01.x, c01.y), s.C[0]);
+    if constexpr (CH == 3) {
+        const float2 c2 = *reinterpret_cast<const float2*>(col + 1);
+        s.C[1] = fma2(nw, make_float2(c01.z, c01.w), s.C[1]);
+        s.C[2] = fma2(nw, c2, s.C[2]);
+    }
+    s.l0 = nw.x < 0.0f ? slot : s.l0;
+    s.l1 = nw.y < 0.0f ? slot : s.l1;
+    s.T.x = a0 ? Tn.x : -fabsf(s.T.x);
+    s.T.y = a1 ? Tn.y : -fabsf(s.T.y);
+}
+
+// Blends a staged batch.  HARD: alphas are clamped, positive powers skipped and
+// (odd) the two Gaussians of a pair voted on apart, so that a colour that is
+// not finite stays with the blocks that blend it.
+template <int CH, bool HARD, int SLOTS>
+__device__ __forceinline__ void blend_batch(FwdPixels<CH>& s, const Stage<SLOTS>& st, int ns,
+                                            float2 nx0, float2 nx1, float2 ny, bool odd) {
+    for (int p = 0; 2 * p < ns; ++p) {
+        const float4 A = st.par[p][0], B = st.par[p][1], D = st.par[p][2];
+        const float2 dy = add2(make_float2(A.z, A.w), ny);
+        const float2 cdd = mul2(make_float2(D.x, D.y), mul2(dy, dy));
+        const float2 gx = make_float2(A.x, A.y), a = make_float2(B.x, B.y),
+                     nb = make_float2(B.z, B.w), no = make_float2(D.z, D.w);
+        PairAlpha e0 = pair_alpha(add2(gx, nx0), dy, cdd, a, nb, no);
+        PairAlpha e1 = pair_alpha(add2(gx, nx1), dy, cdd, a, nb, no);
+        if (HARD) {
+            e0.noG = tame(e0);
+            e1.noG = tame(e1);
+        }
+        const bool hA0 = e0.noG.x <= -kAlphaMin, hA1 = e1.noG.x <= -kAlphaMin;
+        const bool hB0 = e0.noG.y <= -kAlphaMin, hB1 = e1.noG.y <= -kAlphaMin;
+        // one vote for the pair: that a pixel still accumulating blends either
+        if (!__any_sync(kAll,
+                        ((hA0 || hB0) && s.T.x > 0.0f) || ((hA1 || hB1) && s.T.y > 0.0f))) {
+            if (!__any_sync(kAll, fmaxf(s.T.x, s.T.y) > 0.0f)) return;
+            continue;
+        }
+        bool do_a = true, do_b = true;
+        if (HARD && odd) {
+            do_a = __any_sync(kAll, (hA0 && s.T.x > 0.0f) || (hA1 && s.T.y > 0.0f));
+            do_b = __any_sync(kAll, (hB0 && s.T.x > 0.0f) || (hB1 && s.T.y > 0.0f));
+        }
+        if (do_a)
+            blend_one<CH>(s, make_float2(hA0 ? e0.noG.x : 0.0f, hA1 ? e1.noG.x : 0.0f),
+                          st.col[2 * p], 2 * p);
+        if (do_b)
+            blend_one<CH>(s, make_float2(hB0 ? e0.noG.y : 0.0f, hB1 ? e1.noG.y : 0.0f),
+                          st.col[2 * p + 1], 2 * p + 1);
+    }
+}
+
+template <int CH, bool CULL, int SLOTS, int RING>
+__device__ __forceinline__ void fwd_block(const ViewTable& vt, const TileCtx& tc, int bx, int by,
+                                          Feeder<SLOTS, RING>& fd, float bg0, float bg1, float bg2,
+                                          float* __restrict__ images, float* __restrict__ final_T,
+                                          int32_t* __restrict__ last_idx) {
+    const int lane = threadIdx.x & 31;
+    const int lx = bx + 2 * (lane & 3), ly = by + (lane >> 2);
+    const int px = tc.tx0 + lx, py = tc.ty0 + ly;
+    const float2 nx0 = dup(-(float)lx), nx1 = dup(-(float)(lx + 1)), ny = dup(-(float)ly);
+    const bool in0 = py < tc.height && px < tc.width, in1 = py < tc.height && px + 1 < tc.width;
+    FwdPixels<CH> s;
+    s.T = make_float2(in0 ? 1.0f : -1.0f, in1 ? 1.0f : -1.0f);
+#pragma unroll
+    for (int c = 0; c < CH; ++c) s.C[c] = dup(0.0f);
+    int last0 = 0, last1 = 0;
+    const int total = (int)(tc.end - tc.begin), begin = (int)tc.begin;
+    const int chunks = (total + kChunk - 1) / kChunk;
+    auto pos = [&](int c) {
+        const int i = c * kChunk + lane;
+        return i < total ? begin + i : -1;
+    };
+    fd.start(pos, lane);
+    int c = 0;
+    bool alive = __any_sync(kAll, in0 || in1);
+    while (c < chunks && alive) {
+        int ns = 0;
+        do {
+            ns += __popc(fd.template stage<CH, CULL, true>(pos, c, ns, lane, (float)tc.tx0,
+                                                           (float)tc.ty0, (float)bx, (float)by,
+                                                           begin));
+            ++c;
+        } while (ns <= SLOTS - kChunk && c < chunks);
+        fd.pad(ns, lane);
+        __syncwarp();
+        s.l0 = s.l1 = -1;
+        if (fd.hard(ns, lane) || fd.odd)
+            blend_batch<CH, true>(s, *fd.st, ns, nx0, nx1, ny, fd.odd);
+        else
+            blend_batch<CH, false>(s, *fd.st, ns, nx0, nx1, ny, false);
+        constexpr int kTag = CH == 3 ? 6 : 2;
+        if (s.l0 >= 0)
+            last0 = __float_as_int(reinterpret_cast<const float*>(fd.st->col[s.l0])[kTag]) + 1;
+        if (s.l1 >= 0)
+            last1 = __float_as_int(reinterpret_cast<const float*>(fd.st->col[s.l1])[kTag]) + 1;
+        alive = __any_sync(kAll, fmaxf(s.T.x, s.T.y) > 0.0f);
+    }
+    cp_async_wait_all();  // nothing may still be landing in shared memory
+    __syncwarp();
+    if (!in0) return;
+    s.T = make_float2(fabsf(s.T.x), fabsf(s.T.y));
+    const int64_t plane = (int64_t)tc.width * tc.height;
+    const int64_t pix = (int64_t)py * tc.width + px;
+    const float bgc[3] = {bg0, bg1, bg2};
+    const float bgg = (bg0 + bg1 + bg2) * (1.0f / 3.0f);
+#pragma unroll
+    for (int ch = 0; ch < CH; ++ch) {
+        float* o = images + tc.val_base + ch * plane + pix;
+        const float b = CH == 3 ? bgc[ch] : bgg;
+        o[0] = fmaf(s.T.x, b, -s.C[ch].x);
+        if (in1) o[1] = fmaf(s.T.y, b, -s.C[ch].y);
+    }
+    final_T[tc.pix_base + pix] = s.T.x;
+    last_idx[tc.pix_base + pix] = last0;
+    if (in1) {
+        final_T[tc.pix_base + pix + 1] = s.T.y;
+        last_idx[tc.pix_base + pix + 1] = last1;
+    }
+}
+
+// A warp's next block: a slot of the heavy-first tile order times the tile's
+// blocks, from the launch's queue counter.
+__device__ __forceinline__ int next_slot(uint32_t* queue) {
+    int s = 0;
+    if ((threadIdx.x & 31) == 0) s = (int)atomicAdd(queue, 1u);
+    return __shfl_sync(kAll, s, 0);
+}
+
+constexpr int kSlots = 2 * kChunk;
+template <bool CULL>
+constexpr int kRing = CULL ? 2 : 1;
+
+template <bool CULL>
+struct FwdShared {
+    Stage<kSlots> st;
+    float4 raw[kRing<CULL> * kChunk * 3];
+};
+
+template <bool CULL>
+__global__ void __launch_bounds__(32 * kWarps, 8)
+k_blocks_fwd(ViewTable vt, const uint32_t* __restrict__ ranges,
+             const uint32_t* __restrict__ order, const uint32_t* __restrict__ ivals,
+             const uint32_t* __restrict__ gid_of, const float4* __restrict__ rec, int log2_bx,
+             int log2_blocks, int total_blocks, uint32_t* queue, float bg0, float bg1, float bg2,
+             float* __restrict__ images, float* __restrict__ final_T,
+             int32_t* __restrict__ last_idx) {
+    __shared__ FwdShared<CULL> sh[kWarps];
+    FwdShared<CULL>& my = sh[threadIdx.x >> 5];
+    Feeder<kSlots, kRing<CULL>> fd;
+    fd.raw = my.raw;
+    fd.st = &my.st;
+    fd.ivals = ivals;
+    fd.gid_of = gid_of;
+    fd.rec = rec;
+    for (;;) {
+        const int slot = next_slot(queue);
+        if (slot >= total_blocks) break;
+        const TileCtx tc = tile_ctx(vt, ranges, (int)order[slot >> log2_blocks]);
+        const int sub = slot & ((1 << log2_blocks) - 1);
+        const int bx = (sub & ((1 << log2_bx) - 1)) * kBlock, by = (sub >> log2_bx) * kBlock;
+        if (tc.tx0 + bx >= tc.width || tc.ty0 + by >= tc.height) continue;
+        if (tc.channels == 3)
+            fwd_block<3, CULL>(vt, tc, bx, by, fd, bg0, bg1, bg2, images, final_T, last_idx);
+        else
+            fwd_block<1, CULL>(vt, tc, bx, by, fd, bg0, bg1, bg2, images, final_T, last_idx);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Adjoint.
+// ---------------------------------------------------------------------------
+
+// Rows of the window in shared memory: Gaussian r's lane e (its two pixels)
+// holds {dp, dp', w, w'} (both negated) at row_slot(r, e); the order within a row makes
+// the reads below free of bank conflicts.
+constexpr int kRows = 8;
+__device__ __forceinline__ int row_slot(int r, int e) {
+    const int c = e >> 3;
+    return r * 32 + (c << 3) + ((e & 7) ^ c ^ ((r & 1) << 2));
+}
+// ... and {|h_x|, |h_y|} of the density statistic, two lanes per float4.
+__device__ __forceinline__ int abs_slot(int r, int e2) {
+    const int c = e2 >> 2;
+    return r * 16 + (c << 2) + ((e2 & 3) ^ ((c >> 1) | ((r & 1) << 1)));
+}
+
+// x = lo - nhi: nhi, the negated high part, exact in TF32, lo up to its last two bits.
+__device__ __forceinline__ void split_tf32(float2 x, uint32_t (&nhi)[2], uint32_t (&lo)[2]) {
+    nhi[0] = (__float_as_uint(x.x) & 0xffffe000u) ^ 0x80000000u;
+    nhi[1] = (__float_as_uint(x.y) & 0xffffe000u) ^ 0x80000000u;
+    const float2 l = add2(x, make_float2(__uint_as_float(nhi[0]), __uint_as_float(nhi[1])));
+    lo[0] = __float_as_uint(l.x);
+    lo[1] = __float_as_uint(l.y);
+}
+__device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                         uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, "
+        "{%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <bool CULL, bool ABS>
+struct BwdShared {
+    float4 win[(kRows + 1) * 32];
+    float4 habs[ABS ? (kRows + 1) * 16 : 1];
+    Stage<kSlots> st;
+    float4 raw[kRing<CULL> * kChunk * 3];
+    int row_of[kRows + 4];  // the window rows' slots in the stage
+};
+
+// Monomials about the block's centre, as the B operand: entry [s][lane] holds
+// those of the two pixels that k-step s takes from lane 8 (lane % 4) + s; the
+// monomial is the lane's column lane / 4 (1, x, y, x^2, xy, y^2, 0, 0).
+struct Monomials {
+    float2 b[8][32];
+};
+__device__ __forceinline__ float monomial(int n, float x, float y) {
+    return n == 0 ? 1.0f : n == 1 ? x : n == 2 ? y : n == 3 ? x * x : n == 4 ? x * y
+           : n == 5 ? y * y : 0.0f;
+}
+
+struct BwdOut {
+    float* __restrict__ grad2d;
+    float* __restrict__ absgrad;
+    float* __restrict__ partial;
+};
+
+// Sums the window's rows over the block and sends the gradients of the
+// Gaussians of its first `rows` rows on their way.  row_of: the rows' slots in
+// the stage.  gb: dL/dC as the B operand.
+template <int CH, bool ABS, int SLOTS>
+__device__ __forceinline__ void flush_window(const float4* win, const float4* habs,
+                                             const int* row_of, const Stage<SLOTS>& st,
+                                             const Monomials& mono, const uint32_t (&gb)[8][2],
+                                             int rows, float cx, float cy, const BwdOut& out) {
+    const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
+    __syncwarp();
+    const int slot = r < rows ? row_of[r] : 0;
+    float m[4] = {0.f, 0.f, 0.f, 0.f}, k[4] = {0.f, 0.f, 0.f, 0.f};
+    float m2[4] = {0.f, 0.f, 0.f, 0.f};  // every other k-step's moments: half as long a chain of sums
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+        const float4 q = win[row_slot(r, 8 * c + s)];
+        const float2 b = mono.b[s][lane];
+        uint32_t h[2], l[2];
+        split_tf32(make_float2(q.x, q.y), h, l);
+        mma_tf32(s & 1 ? m2 : m, h[0], l[0], h[1], l[1], __float_as_uint(b.x),
+                 __float_as_uint(b.y));
+        split_tf32(make_float2(q.z, q.w), h, l);
+        mma_tf32(k, h[0], l[0], h[1], l[1], gb[s][0], gb[s][1]);
+    }
+    if constexpr (ABS) {
+        // the two magnitude sums, into columns 6 and 7
+        const uint32_t b6 = r == 6 ? __float_as_uint(1.0f) : 0u;
+        const uint32_t b7 = r == 7 ? __float_as_uint(1.0f) : 0u;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const float4 q = habs[abs_slot(r, 4 * c + s)];
+            uint32_t h[2], l[2];
+            split_tf32(make_float2(q.x, q.z), h, l);
+            mma_tf32(m, h[0], l[0], h[1], l[1], b6, b6);
+            split_tf32(make_float2(q.y, q.w), h, l);
+            mma_tf32(m, h[0], l[0], h[1], l[1], b7, b7);
+        }
+    }
+    __syncwarp();  // the window may be written again
+    // high and low rows; the moments of row r sit in its four lanes, two each
+    const float e0 = (m[2] + m2[2]) - (m[0] + m2[0]), e1 = (m[3] + m2[3]) - (m[1] + m2[1]);
+    const float col = (k[0] - k[2]) + (k[1] - k[3]);
+    const int base = lane & ~3;
+    const float A0 = -__shfl_sync(kAll, e0, base), Sx = -__shfl_sync(kAll, e1, base);
+    const float Sy = -__shfl_sync(kAll, e0, base + 1), Sxx = -__shfl_sync(kAll, e1, base + 1);
+    const float Sxy = -__shfl_sync(kAll, e0, base + 2), Syy = -__shfl_sync(kAll, e1, base + 2);
+    if (r >= rows) return;
+    const float* f = reinterpret_cast<const float*>(&st.par[slot >> 1][0]) + (slot & 1);
+    const float mx = f[0] - cx, my = f[2] - cy, nb = f[6], no = f[10];
+    const float na = 2.0f * f[4], nc = 2.0f * f[8];
+    constexpr int kTag = CH == 3 ? 6 : 2;
+    const uint32_t id =
+        __float_as_uint(reinterpret_cast<const float*>(st.col[slot])[kTag]);
+    // moments about the mean
+    const float A1 = fmaf(mx, A0, -Sx), A2 = fmaf(my, A0, -Sy);
+    const float A3 = fmaf(mx, A1 - Sx, Sxx);
+    const float A4 = fmaf(mx, A2, fmaf(-my, Sx, Sxy));
+    const float A5 = fmaf(my, A2 - Sy, Syy);
+    // lane c writes components c, 4 + c (c < 2) and 6 + c (c < CH)
+    const float v0 = c == 0   ? fmaf(nb, A2, na * A1)
+                     : c == 1 ? fmaf(nb, A1, nc * A2)
+                     : c == 2 ? -0.5f * A3
+                              : -A4;
+    // A0 / o by the reciprocal and one correction of the quotient
+    const float ro = rcp_approx(no), qo = -A0 * ro;
+    const float v1 = c == 0 ? -0.5f * A5 : fmaf(fmaf(-qo, no, -A0), ro, qo);
+    if (out.partial) {
+        float* o = out.partial + (size_t)id * 11;
+        o[c] = v0;
+        if (c < 2) o[4 + c] = v1;
+        if (c < CH) o[6 + c] = col;
+        if (ABS && c == 3) {
+            o[9] = e0;
+            o[10] = e1;
+        }
+    } else {
+        float* o = out.grad2d + (size_t)id * kGrad2d;
+        if (v0 != 0.0f) atomicAdd(o + c, v0);
+        if (c < 2 && v1 != 0.0f) atomicAdd(o + 4 + c, v1);
+        if (c < CH && col != 0.0f) atomicAdd(o + 6 + c, col);
+        if (ABS && c == 3) {
+            float* h = out.absgrad + (size_t)id * 2;
+            if (e0 != 0.0f) atomicAdd(h, e0);
+            if (e1 != 0.0f) atomicAdd(h + 1, e1);
+        }
+    }
+}
+
+template <int CH>
+struct BwdPixels {
+    float2 T, nS, g[CH];  // T behind the current Gaussian; -dL/dC . (colour behind); dL/dC
+};
+
+// One Gaussian's adjoint at the lane's two pixels into a row of the window
+// (win, habs: the lane's places in it).  na: -alpha where the Gaussian counts
+// at the pixel, else 0, which leaves the pixel's state as it is; nG: -o G where
+// alpha = o G, 0 where alpha is clamped (and passes no gradient).
+template <int CH, bool ABS>
+__device__ __forceinline__ void adjoint_one_block(BwdPixels<CH>& s, float2 na, float2 nG,
+                                                  const float4* col, float4* win, float2* habs,
+                                                  float ha, float nb, float hc, float dx0,
+                                                  float dx1, float dy) {
+    const float2 inv = make_float2(rcp_approx(1.0f + na.x), rcp_approx(1.0f + na.y));
+    s.T = mul2(s.T, inv);
+    const float2 nw = mul2(na, s.T);
+    const float4 c01 = col[0];
+    float2 gc = mul2(s.g[0], make_float2(c01.x, c01.y));
+    if constexpr (CH == 3) {
+        const float2 c2 = *reinterpret_cast<const float2*>(col + 1);
+        gc = fma2(s.g[1], make_float2(c01.z, c01.w), gc);
+        gc = fma2(s.g[2], c2, gc);
+    }
+    const float2 dal = fma2(s.T, gc, mul2(inv, s.nS));
+    s.nS = fma2(nw, gc, s.nS);
+    const float2 ndp = mul2(nG, dal);
+    *win = make_float4(ndp.x, ndp.y, nw.x, nw.y);
+    if constexpr (ABS) {
+        // each pixel's own contribution to dL/dmean2d, by magnitude
+        const float a = -2.0f * ha, c = -2.0f * hc;
+        const float hx = fabsf(ndp.x * fmaf(a, dx0, -nb * dy)) + fabsf(ndp.y * fmaf(a, dx1, -nb * dy));
+        const float hy = fabsf(ndp.x * fmaf(-nb, dx0, c * dy)) + fabsf(ndp.y * fmaf(-nb, dx1, c * dy));
+        *habs = make_float2(hx, hy);
+    }
+}
+
+// The adjoint of a staged batch.  HARD: alphas are clamped and positive powers
+// skipped.
+template <int CH, bool ABS, bool HARD, int SLOTS>
+__device__ __forceinline__ void adjoint_batch(
+    BwdPixels<CH>& s, const Stage<SLOTS>& st, int ns, int from0, int from1, int checked,
+    float2 nx0, float2 nx1, float2 ny, float4* win, float4* habs, int* row_of,
+    const Monomials& mono, const uint32_t (&gb)[8][2], float cx, float cy, const BwdOut& out) {
+    const int lane = threadIdx.x & 31;
+    // the lane's place in row 0 and what takes it from one row to the next
+    const int place0 = row_slot(0, lane), hop = 32, flip = 4;
+    int rows = 0;  // rows of the window in use
+    int place = place0;
+    float limA0 = -kAlphaMin, limA1 = -kAlphaMin, limB0 = -kAlphaMin, limB1 = -kAlphaMin;
+    for (int p = 0;;) {
+        const bool end = 2 * p >= ns;
+        if (rows >= kRows || (end && rows > 0)) {
+            flush_window<CH, ABS>(win, habs, row_of, st, mono, gb, min(rows, kRows), cx, cy, out);
+            rows = max(rows - kRows, 0);
+            place = place0;
+            if (rows > 0) {  // the ninth row becomes the first
+                win[place0] = win[row_slot(kRows, lane)];
+                if (ABS && lane < 16) habs[abs_slot(0, lane)] = habs[abs_slot(kRows, lane)];
+                if (lane == 0) row_of[0] = row_of[kRows];
+                place = (place0 + hop) ^ flip;
+                __syncwarp();
+            }
+        }
+        if (end) {
+            if (rows == 0) break;
+            continue;
+        }
+        const float4 A = st.par[p][0], B = st.par[p][1], D = st.par[p][2];
+        const float2 dy = add2(make_float2(A.z, A.w), ny);
+        const float2 cdd = mul2(make_float2(D.x, D.y), mul2(dy, dy));
+        const float2 gx = make_float2(A.x, A.y), a = make_float2(B.x, B.y),
+                     nb = make_float2(B.z, B.w), no = make_float2(D.z, D.w);
+        const float2 dx0 = add2(gx, nx0), dx1 = add2(gx, nx1);
+        const PairAlpha e0 = pair_alpha(dx0, dy, cdd, a, nb, no);
+        const PairAlpha e1 = pair_alpha(dx1, dy, cdd, a, nb, no);
+        if (p <= checked) {  // (one more than needed: puts the limits back)
+            limA0 = 2 * p >= from0 ? -kAlphaMin : -2.0f;
+            limA1 = 2 * p >= from1 ? -kAlphaMin : -2.0f;
+            limB0 = 2 * p + 1 >= from0 ? -kAlphaMin : -2.0f;
+            limB1 = 2 * p + 1 >= from1 ? -kAlphaMin : -2.0f;
+        }
+        float2 n0 = e0.noG, n1 = e1.noG;
+        if (HARD) {
+            n0 = tame(e0);
+            n1 = tame(e1);
+        }
+        const bool hA0 = n0.x <= limA0, hA1 = n1.x <= limA1;
+        const bool hB0 = n0.y <= limB0, hB1 = n1.y <= limB1;
+        const bool any_b = __any_sync(kAll, hB0 || hB1);
+        if (__any_sync(kAll, hA0 || hA1)) {
+            const float2 na = make_float2(hA0 ? n0.x : 0.0f, hA1 ? n1.x : 0.0f);
+            float2 nG = na;
+            if (HARD)
+                nG = make_float2(e0.noG.x > -kAlphaMax ? na.x : 0.0f,
+                                 e1.noG.x > -kAlphaMax ? na.y : 0.0f);
+            adjoint_one_block<CH, ABS>(
+                s, na, nG, st.col[2 * p], win + place,
+                reinterpret_cast<float2*>(habs + abs_slot(rows, lane >> 1)) + (lane & 1), a.x,
+                nb.x, D.x, dx0.x, dx1.x, dy.x);
+            if (lane == 0) row_of[rows] = 2 * p;
+            ++rows;  // at most eight now
+            place = (place + hop) ^ flip;
+        }
+        if (any_b) {
+            const float2 na = make_float2(hB0 ? n0.y : 0.0f, hB1 ? n1.y : 0.0f);
+            float2 nG = na;
+            if (HARD)
+                nG = make_float2(e0.noG.y > -kAlphaMax ? na.x : 0.0f,
+                                 e1.noG.y > -kAlphaMax ? na.y : 0.0f);
+            adjoint_one_block<CH, ABS>(
+                s, na, nG, st.col[2 * p + 1], win + place,
+                reinterpret_cast<float2*>(habs + abs_slot(rows, lane >> 1)) + (lane & 1), a.y,
+                nb.y, D.y, dx0.y, dx1.y, dy.y);
+            if (lane == 0) row_of[rows] = 2 * p + 1;
+            ++rows;
+            place = (place + hop) ^ flip;
+        }
+        ++p;
+    }
+}
+
+template <int CH, bool CULL, bool ABS, int SLOTS, int RING>
+__device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
+                                          Feeder<SLOTS, RING>& fd, float4* win, float4* habs,
+                                          int* row_of, const Monomials& mono, float bg0, float bg1, float bg2,
+                                          const float* __restrict__ final_T,
+                                          const int32_t* __restrict__ last_idx,
+                                          const float* __restrict__ dL, const BwdOut& out) {
+    const int lane = threadIdx.x & 31;
+    const int lx = bx + 2 * (lane & 3), ly = by + (lane >> 2);
+    const int px = tc.tx0 + lx, py = tc.ty0 + ly;
+    const bool in0 = py < tc.height && px < tc.width, in1 = py < tc.height && px + 1 < tc.width;
+    const int64_t plane = (int64_t)tc.width * tc.height;
+    const int64_t pix = (int64_t)py * tc.width + px;
+    int last0 = 0, last1 = 0;
+    if (in0) last0 = last_idx[tc.pix_base + pix];
+    if (in1) last1 = last_idx[tc.pix_base + pix + 1];
+    const int top = (int)__reduce_max_sync(kAll, (unsigned)max(last0, last1));
+    if (top == 0) return;
+    const int begin = (int)tc.begin;
+    const int chunks = (top + kChunk - 1) / kChunk;
+    // chunk c, lane i: the list from its last blended entry on, backwards
+    auto pos = [&](int c) {
+        const int i = top - 1 - (c * kChunk + lane);
+        return i >= 0 ? begin + i : -1;
+    };
+    fd.start(pos, lane);
+    BwdPixels<CH> s;
+    s.T = make_float2(in0 ? final_T[tc.pix_base + pix] : 1.0f,
+                      in1 ? final_T[tc.pix_base + pix + 1] : 1.0f);
+    const float bgc[3] = {bg0, bg1, bg2};
+    const float bgg = (bg0 + bg1 + bg2) * (1.0f / 3.0f);
+    float2 gb2 = dup(0.0f);
+#pragma unroll
+    for (int ch = 0; ch < CH; ++ch) {
+        const float* d = dL + tc.val_base + ch * plane + pix;
+        s.g[ch] = make_float2(in0 ? d[0] : 0.0f, in1 ? d[1] : 0.0f);
+        gb2 = fma2(s.g[ch], dup(CH == 3 ? bgc[ch] : bgg), gb2);
+    }
+    s.nS = mul2(s.T, make_float2(-gb2.x, -gb2.y));  // minus the background seen through T_final
+    // dL/dC as the B operand: column n = lane / 4 holds the high (n even) or
+    // low part of channel n / 2
+    uint32_t gb[8][2];
+    {
+        float2* x = reinterpret_cast<float2*>(win);
+#pragma unroll
+        for (int ch = 0; ch < CH; ++ch) x[ch * 32 + lane] = s.g[ch];
+        __syncwarp();
+        const int n = lane >> 2, ch = n >> 1;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float2 v = ch < CH ? x[ch * 32 + 8 * (lane & 3) + k] : dup(0.0f);
+            uint32_t h[2], l[2];
+            split_tf32(v, h, l);
+            gb[k][0] = n & 1 ? l[0] : h[0] ^ 0x80000000u;
+            gb[k][1] = n & 1 ? l[1] : h[1] ^ 0x80000000u;
+        }
+        __syncwarp();
+    }
+    const float2 nx0 = dup(-(float)lx), nx1 = dup(-(float)(lx + 1)), ny = dup(-(float)ly);
+    const float cx = (float)bx + 3.5f, cy = (float)by + 3.5f;
+    for (int c = 0; c < chunks;) {
+        // from0, from1: the first slot of this batch within the pixel's part of the list
+        int ns = 0, from0 = 0, from1 = 0;
+        do {
+            const unsigned mask = fd.template stage<CH, CULL, false>(
+                pos, c, ns, lane, (float)tc.tx0, (float)tc.ty0, (float)bx, (float)by, begin);
+            const int hi = top - c * kChunk;  // entries behind the pixel's last: hi - last
+            const int d0 = min(max(hi - last0, 0), 32), d1 = min(max(hi - last1, 0), 32);
+            from0 += __popc(mask & (unsigned)((1ull << d0) - 1ull));
+            from1 += __popc(mask & (unsigned)((1ull << d1) - 1ull));
+            ns += __popc(mask);
+            ++c;
+        } while (ns <= SLOTS - kChunk && c < chunks);
+        fd.pad(ns, lane);
+        __syncwarp();
+        // pairs before this one hold slots beyond some pixel's part of the list
+        const int checked = ((int)__reduce_max_sync(kAll, (unsigned)max(from0, from1)) + 1) >> 1;
+        if (fd.hard(ns, lane))
+            adjoint_batch<CH, ABS, true>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny, win,
+                                         habs, row_of, mono, gb, cx, cy, out);
+        else
+            adjoint_batch<CH, ABS, false>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny, win,
+                                          habs, row_of, mono, gb, cx, cy, out);
+        __syncwarp();  // the stage has been read
+    }
+    cp_async_wait_all();
+    __syncwarp();
+}
+
+template <bool CULL, bool ABS>
+__global__ void __launch_bounds__(32 * kWarps, 5)
+k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
+             const uint32_t* __restrict__ order, const uint32_t* __restrict__ ivals,
+             const uint32_t* __restrict__ gid_of, const float4* __restrict__ rec, int log2_bx,
+             int log2_blocks, int total_blocks, uint32_t* queue, float bg0, float bg1, float bg2,
+             const float* __restrict__ final_T, const int32_t* __restrict__ last_idx,
+             const float* __restrict__ dL, BwdOut out) {
+    extern __shared__ float4 smem[];
+    Monomials& mono = *reinterpret_cast<Monomials*>(smem);
+    BwdShared<CULL, ABS>& my = reinterpret_cast<BwdShared<CULL, ABS>*>(
+        smem + sizeof(Monomials) / sizeof(float4))[threadIdx.x >> 5];
+    for (int i = threadIdx.x; i < 8 * 32; i += blockDim.x) {
+        const int s = i >> 5, l = i & 31, e = 8 * (l & 3) + s;
+        const float x = (float)(2 * (e & 3)) - 3.5f, y = (float)(e >> 2) - 3.5f;
+        mono.b[s][l] = make_float2(monomial(l >> 2, x, y), monomial(l >> 2, x + 1.0f, y));
+    }
+    __syncthreads();
+    Feeder<kSlots, kRing<CULL>> fd;
+    fd.raw = my.raw;
+    fd.st = &my.st;
+    fd.ivals = ivals;
+    fd.gid_of = gid_of;
+    fd.rec = rec;
+    for (;;) {
+        const int slot = next_slot(queue);
+        if (slot >= total_blocks) break;
+        const TileCtx tc = tile_ctx(vt, ranges, (int)order[slot >> log2_blocks]);
+        const int sub = slot & ((1 << log2_blocks) - 1);
+        const int bx = (sub & ((1 << log2_bx) - 1)) * kBlock, by = (sub >> log2_bx) * kBlock;
+        if (tc.channels == 3)
+            bwd_block<3, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, my.row_of, mono, bg0, bg1, bg2, final_T,
+                                    last_idx, dL, out);
+        else
+            bwd_block<1, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, my.row_of, mono, bg0, bg1, bg2, final_T,
+                                    last_idx, dL, out);
+    }
+}
+
+// CTAs of a launch over `total` blocks: the resident ones, but no more than
+// leave each warp per_warp2 / 2 blocks (and at least two per SM).  A warp's
+// share of its SM shrinks with every other warp there, and a launch is not over
+// before its longest list, which one warp walks alone: where there are few
+// blocks, fewer warps that run faster end sooner.  Forward (8 halves),
+// at 8 / 5 / 3 / 2 CTAs per SM: 113640 blocks 632 / 696 / 897 / 1197 us, 12750
+// blocks 148 / 134 / 150 / 189, 4800 blocks 56 / 55 / 46 / 39.  Adjoint (5 halves)
+// at 5 / 3 / 2: 113640 blocks 1429 / 1798 / 2486, 12750 blocks 261 / 306 / 408, 4800
+// blocks 95 / 86 / 91.
+int launch_ctas(const void* kern, size_t smem, int total, int per_warp2) {
+    const int resident = persistent_blocks(kern, 32 * kWarps, smem, kWarps, total);
+    const int sms = sm_count();
+    if (resident < 0 || sms <= 0) return -1;
+    const int per_sm = max(2, (int)(2ll * total / ((long long)sms * kWarps * per_warp2)));
+    return per_sm < resident / sms ? per_sm * sms : resident;
+}
+
+int ilog2(int x) {
+    int l = 0;
+    while ((1 << (l + 1)) <= x) ++l;
+    return l;
+}
+
+}  // namespace
+
+// The block kernels take every tile that is whole 8x8 blocks; with a
+// deterministic adjoint only the 8x8 tile itself, whose (Gaussian, tile)
+// pairs one warp sums (the larger tiles' pairs would be split over warps).
+bool blocks_fit(const Plan* p) {
+    if (p->cfg.tile_w % kBlock || p->cfg.tile_h % kBlock) return false;
+    return !p->cfg.deterministic || (p->cfg.tile_w == kBlock && p->cfg.tile_h == kBlock);
+}
+
+gs_status launch_blocks_fwd(const Plan* p, const uint32_t* vals, void* ws, float* images,
+                            float* final_T, int32_t* last_idx, cudaStream_t st) {
+    const int log2_bx = ilog2(p->cfg.tile_w / kBlock);
+    const int log2_blocks = log2_bx + ilog2(p->cfg.tile_h / kBlock);
+    const bool cull = log2_blocks > 0 || !p->vt.tight_rect;
+    const int total = p->total_tiles << log2_blocks;
+    auto* kern = cull ? k_blocks_fwd<true> : k_blocks_fwd<false>;
+    const int blocks = launch_ctas((const void*)kern, 0, total, 8);
+    if (blocks < 0) return GS_ERR_CUDA;
+    uint32_t* queue = buf<uint32_t>(p, ws, B_TILE_QUEUE);
+    if (cudaMemsetAsync(queue, 0, sizeof(uint32_t), st) != cudaSuccess) return GS_ERR_CUDA;
+    kern<<<blocks, 32 * kWarps, 0, st>>>(
+        p->vt, cbuf<uint32_t>(p, ws, GS_BUF_RANGES), cbuf<uint32_t>(p, ws, B_TILE_ORDER), vals,
+        p->cfg.deterministic ? cbuf<uint32_t>(p, ws, B_GID_OF) : nullptr,
+        cbuf<float4>(p, ws, GS_BUF_PROJ), log2_bx, log2_blocks, total, queue, p->cfg.bg[0],
+        p->cfg.bg[1], p->cfg.bg[2], images, final_T, last_idx);
+    return launch_status();
+}
+
+gs_status launch_blocks_bwd(const Plan* p, const uint32_t* vals, void* ws, const float* final_T,
+                            const int32_t* last_idx, const float* dL, cudaStream_t st) {
+    const int log2_bx = ilog2(p->cfg.tile_w / kBlock);
+    const int log2_blocks = log2_bx + ilog2(p->cfg.tile_h / kBlock);
+    const bool cull = log2_blocks > 0 || !p->vt.tight_rect;
+    const bool abs_stats = p->cfg.density_stats != 0;
+    const int total = p->total_tiles << log2_blocks;
+    auto* kern = cull ? (abs_stats ? k_blocks_bwd<true, true> : k_blocks_bwd<true, false>)
+                      : (abs_stats ? k_blocks_bwd<false, true> : k_blocks_bwd<false, false>);
+    const size_t per_warp =
+        cull ? (abs_stats ? sizeof(BwdShared<true, true>) : sizeof(BwdShared<true, false>))
+             : (abs_stats ? sizeof(BwdShared<false, true>) : sizeof(BwdShared<false, false>));
+    const size_t smem = sizeof(Monomials) + kWarps * per_warp;
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess)
+        return GS_ERR_CUDA;
+    const int blocks = launch_ctas((const void*)kern, smem, total, 5);
+    if (blocks < 0) return GS_ERR_CUDA;
+    uint32_t* queue = buf<uint32_t>(p, ws, B_TILE_QUEUE) + 1;
+    if (cudaMemsetAsync(queue, 0, sizeof(uint32_t), st) != cudaSuccess) return GS_ERR_CUDA;
+    BwdOut out;
+    out.grad2d = buf<float>(p, ws, GS_BUF_GRAD2D);
+    out.absgrad = abs_stats ? buf<float>(p, ws, GS_BUF_ABSGRAD) : nullptr;
+    out.partial = p->cfg.deterministic ? buf<float>(p, ws, B_PARTIAL) : nullptr;
+    kern<<<blocks, 32 * kWarps, smem, st>>>(
+        p->vt, cbuf<uint32_t>(p, ws, GS_BUF_RANGES), cbuf<uint32_t>(p, ws, B_TILE_ORDER), vals,
+        p->cfg.deterministic ? cbuf<uint32_t>(p, ws, B_GID_OF) : nullptr,
+        cbuf<float4>(p, ws, GS_BUF_PROJ), log2_bx, log2_blocks, total, queue, p->cfg.bg[0],
+        p->cfg.bg[1], p->cfg.bg[2], final_T, last_idx, dL, out);
+    return launch_status();
+}
+
+}  // namespace gs

@@ -30,48 +30,10 @@
 //    and leave as nine parallel atomics per Gaussian.
 #include <mutex>
 
-#include "gs_internal.cuh"
+#include "gs_render.cuh"
 
 namespace gs {
 namespace {
-
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_one() {
-    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-}
-
-struct TileCtx {
-    int view, tile_local, tx0, ty0, width, height, channels;
-    int64_t pix_base, val_base;
-    uint32_t begin, end;
-};
-
-__device__ __forceinline__ TileCtx tile_ctx(const ViewTable& vt, const uint32_t* ranges,
-                                            int tile) {
-    TileCtx c;
-    c.view = view_of_tile(vt, tile);
-    const ViewGeom& g = vt.v[c.view];
-    c.tile_local = tile - g.tile_offset;
-    c.tx0 = (c.tile_local % g.tiles_x) * vt.tile_w;
-    c.ty0 = (c.tile_local / g.tiles_x) * vt.tile_h;
-    c.width = g.width;
-    c.height = g.height;
-    c.channels = g.channels;
-    c.pix_base = g.pixel_offset;
-    c.val_base = g.value_offset;
-    c.begin = ranges[2 * tile];
-    c.end = ranges[2 * tile + 1];
-    return c;
-}
 
 // The threads that render one tile: the whole CTA (one tile per CTA), or a
 // single warp (one tile per warp, several tiles per CTA), whose barriers,
@@ -554,14 +516,6 @@ __device__ __forceinline__ int reduce_component(int lane) {
     return idx;
 }
 
-// Reciprocal by the hardware approximation (PTX rcp.approx.ftz.f32, within
-// about one ulp); the argument 1 - alpha lies in [0.01, 1].
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // The pixel adjoint's per-Gaussian work for a lane holding an even number of
 // pixels, in pairs on packed FP32 pair operations: each half is the scalar
 // operation of the one-pixel path in render_bwd_tile on the same operands,
@@ -1035,7 +989,7 @@ static int warp_teams(int tf4) {
 // CTAs of a persistent launch: the resident CTAs of the whole GPU, no more
 // than there are teams' worth of tiles.  The occupancy query runs once per
 // (kernel, shape, device) and is cached.
-static int persistent_blocks(const void* kern, int threads, size_t smem, int tiles_per_block,
+int persistent_blocks(const void* kern, int threads, size_t smem, int tiles_per_block,
                              int total_tiles) {
     struct Entry {
         const void* k;
@@ -1093,11 +1047,12 @@ gs_status launch_render_fwd(const Plan* p, void* ws, float* images, float* final
                             int32_t* last_idx, cudaStream_t st) {
     const int batch = p->cfg.smem_batch;
     const int ppt = p->cfg.pixels_per_thread;
+    const uint32_t* vals =
+        cbuf<uint32_t>(p, ws, (p->tile_passes & 1) ? (int)B_IVAL_B : (int)GS_BUF_TILE_VALUES);
+    if (blocks_fit(p)) return launch_blocks_fwd(p, vals, ws, images, final_T, last_idx, st);
     const RenderShape s = render_shape(p, batch, ppt, false);
     const uint32_t* ranges = cbuf<uint32_t>(p, ws, GS_BUF_RANGES);
     const uint32_t* order = cbuf<uint32_t>(p, ws, B_TILE_ORDER);
-    const uint32_t* vals =
-        cbuf<uint32_t>(p, ws, (p->tile_passes & 1) ? (int)B_IVAL_B : (int)GS_BUF_TILE_VALUES);
     const float4* rec = cbuf<float4>(p, ws, GS_BUF_PROJ);
     const uint32_t* gid_of = p->cfg.deterministic ? cbuf<uint32_t>(p, ws, B_GID_OF) : nullptr;
     uint32_t* queue = buf<uint32_t>(p, ws, B_TILE_QUEUE);
@@ -1116,23 +1071,16 @@ gs_status launch_render_fwd(const Plan* p, void* ws, float* images, float* final
     return launch_status();
 }
 
-gs_status launch_render_bwd_pixels(const Plan* p, void* ws, const float* final_T,
-                                   const int32_t* last_idx, const float* dL, cudaStream_t st) {
+// The pixel adjoint of the tiles the block kernels do not take.
+static gs_status launch_teams_bwd(const Plan* p, const uint32_t* vals, void* ws,
+                                  const float* final_T, const int32_t* last_idx, const float* dL,
+                                  cudaStream_t st) {
     const int batch = p->cfg.smem_batch_bwd;
     const int ppt = p->cfg.pixels_per_thread_bwd;
     const RenderShape s = render_shape(p, batch, ppt, true);
-    float* grad2d = buf<float>(p, ws, GS_BUF_GRAD2D);
-    const uint32_t* ranges = cbuf<uint32_t>(p, ws, GS_BUF_RANGES);
-    const uint32_t* order = cbuf<uint32_t>(p, ws, B_TILE_ORDER);
-    const uint32_t* vals =
-        cbuf<uint32_t>(p, ws, (p->tile_passes & 1) ? (int)B_IVAL_B : (int)GS_BUF_TILE_VALUES);
-    const float4* rec = cbuf<float4>(p, ws, GS_BUF_PROJ);
-    uint32_t* queue = buf<uint32_t>(p, ws, B_TILE_QUEUE) + 1;
     const bool abs_stats = p->cfg.density_stats != 0;
-    float* absgrad = abs_stats ? buf<float>(p, ws, GS_BUF_ABSGRAD) : nullptr;
     const bool det = p->cfg.deterministic != 0;
-    const uint32_t* gid_of = det ? cbuf<uint32_t>(p, ws, B_GID_OF) : nullptr;
-    float* partial = det ? buf<float>(p, ws, B_PARTIAL) : nullptr;
+    uint32_t* queue = buf<uint32_t>(p, ws, B_TILE_QUEUE) + 1;
     auto kern =
         abs_stats
             ? (s.warp ? pick(ppt, k_render_bwd<1, true, true>, k_render_bwd<2, true, true>,
@@ -1146,17 +1094,39 @@ gs_status launch_render_bwd_pixels(const Plan* p, void* ws, const float* final_T
     const int blocks = persistent_blocks((const void*)kern, s.threads, s.smem, s.teams,
                                          p->total_tiles);
     if (blocks < 0) return GS_ERR_CUDA;
-    if (cudaMemsetAsync(grad2d, 0, p->len[GS_BUF_GRAD2D], st) != cudaSuccess) return GS_ERR_CUDA;
     if (cudaMemsetAsync(queue, 0, sizeof(uint32_t), st) != cudaSuccess) return GS_ERR_CUDA;
+    kern<<<blocks, s.threads, s.smem, st>>>(
+        p->vt, cbuf<uint32_t>(p, ws, GS_BUF_RANGES), cbuf<uint32_t>(p, ws, B_TILE_ORDER), vals,
+        det ? cbuf<uint32_t>(p, ws, B_GID_OF) : nullptr, cbuf<float4>(p, ws, GS_BUF_PROJ), batch,
+        s.tf4, p->total_tiles, queue, p->cfg.bg[0], p->cfg.bg[1], p->cfg.bg[2], final_T, last_idx,
+        dL, buf<float>(p, ws, GS_BUF_GRAD2D),
+        abs_stats ? buf<float>(p, ws, GS_BUF_ABSGRAD) : nullptr,
+        det ? buf<float>(p, ws, B_PARTIAL) : nullptr);
+    return launch_status();
+}
+
+gs_status launch_render_bwd_pixels(const Plan* p, void* ws, const float* final_T,
+                                   const int32_t* last_idx, const float* dL, cudaStream_t st) {
+    float* grad2d = buf<float>(p, ws, GS_BUF_GRAD2D);
+    const uint32_t* vals =
+        cbuf<uint32_t>(p, ws, (p->tile_passes & 1) ? (int)B_IVAL_B : (int)GS_BUF_TILE_VALUES);
+    const bool abs_stats = p->cfg.density_stats != 0;
+    float* absgrad = abs_stats ? buf<float>(p, ws, GS_BUF_ABSGRAD) : nullptr;
+    const bool det = p->cfg.deterministic != 0;
+    float* partial = det ? buf<float>(p, ws, B_PARTIAL) : nullptr;
+    if (cudaMemsetAsync(grad2d, 0, p->len[GS_BUF_GRAD2D], st) != cudaSuccess) return GS_ERR_CUDA;
     if (abs_stats &&
         cudaMemsetAsync(absgrad, 0, p->len[GS_BUF_ABSGRAD], st) != cudaSuccess)
         return GS_ERR_CUDA;
     if (det && cudaMemsetAsync(partial, 0, p->len[B_PARTIAL], st) != cudaSuccess)
         return GS_ERR_CUDA;
-    kern<<<blocks, s.threads, s.smem, st>>>(p->vt, ranges, order, vals, gid_of, rec, batch,
-                                            s.tf4, p->total_tiles, queue, p->cfg.bg[0],
-                                            p->cfg.bg[1], p->cfg.bg[2], final_T, last_idx, dL,
-                                            grad2d, absgrad, partial);
+    if (blocks_fit(p)) {
+        const gs_status e = launch_blocks_bwd(p, vals, ws, final_T, last_idx, dL, st);
+        if (e != GS_OK) return e;
+    } else {
+        const gs_status e = launch_teams_bwd(p, vals, ws, final_T, last_idx, dL, st);
+        if (e != GS_OK) return e;
+    }
     if (det) {
         // grid over the plan's capacity; the pair count of the last binning
         // is read on the device
