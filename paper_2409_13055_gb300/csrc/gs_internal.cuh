@@ -15,7 +15,10 @@
 namespace gs {
 
 constexpr uint32_t kPlanMagic = 0x67733330u;  // "gs30"
-constexpr int kOrderBuckets = 33;  // tile-order buckets: bit length of a list length
+constexpr int kOrderSub = 8;  // tile-order buckets per octave of the list length
+constexpr int kOrderBuckets = 33 * kOrderSub;
+constexpr int kCountRows = 160;       // CTAs of the counting tile sort at most
+constexpr int kCountTiles = 24000;  // tiles it takes at most (their counters are shared memory)
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kSortThreads = 256;
@@ -61,6 +64,8 @@ enum PrivBuf {
     B_OFFSETS,  // [V*n + 1] instance offsets of the entries in depth order
     B_TILE_ORDER,  // [total_tiles] render order of the tiles, longest lists first;
                    // then 2 x kOrderBuckets words of scratch for building it
+    B_TILE_COUNTS,  // counting tile sort: [kCountRows][tiles] u32 counts per CTA, then their
+                    // starts within the tile; then [tiles] list lengths
     B_TILE_QUEUE,  // [2] u32 next-tile counters of the forward and backward render
     B_GID_OF,      // [instance_capacity] u32 (view*n + index) of each emitted instance
                    // (deterministic plans: the sort then carries emission positions)
@@ -404,6 +409,10 @@ constexpr float kTMin = 1e-4f;
 gs_status launch_project(const Plan* p, const gs_map* map, const gs_view* views_dev, void* ws,
                          cudaStream_t st);
 gs_status launch_bin_sort(const Plan* p, int32_t n, void* ws, cudaStream_t st);
+bool depth_small_fits(const Plan* p, int32_t n);
+bool tiles_fit(const Plan* p);
+gs_status launch_tiles(const Plan* p, int32_t n, void* ws, cudaStream_t st);
+gs_status launch_depth_small(const Plan* p, int32_t n, void* ws, cudaStream_t st);
 gs_status launch_render_fwd(const Plan* p, void* ws, float* images, float* final_T,
                             int32_t* last_idx, cudaStream_t st);
 gs_status launch_loss(const Plan* p, const float* images, const float* targets, float lambda,

@@ -24,6 +24,8 @@ namespace {
 
 constexpr int kWarps = kSortThreads / 32;
 constexpr int kGridPerSm = 8;  // CTAs per SM of the grid-stride kernels
+constexpr int kTailBuckets = 33;  // bit length of a list length
+static_assert(kTailBuckets <= kOrderBuckets, "they share the order's scratch");
 constexpr uint32_t kCulledKey = 0xFFFFFFFFu;  // depth key of a culled pair (never a depth)
 
 __device__ __forceinline__ uint32_t active_count(const uint32_t* count_dev, uint32_t count_host) {
@@ -290,13 +292,13 @@ k_scan_offsets(const uint32_t* __restrict__ order, const uint32_t* __restrict__ 
         s += t[k];
     }
     uint32_t tot;
-    uint32_t o = block_exclusive_scan(s, wt, tot) +
-                 (uint32_t)min(pre, (unsigned long long)0xFFFFFFFFu);
+    unsigned long long o = pre + block_exclusive_scan(s, wt, tot);
+    auto word = [](unsigned long long x) { return (uint32_t)min(x, 0xFFFFFFFFull); };
     for (int k = 0; k < kScanItems; ++k) {
         const uint32_t i = start + threadIdx.x * kScanItems + k;
         if (i < count) {
-            off[i] = o;
-            if (i + 1 == count) off[count] = o + t[k];  // the total
+            off[i] = word(o);
+            if (i + 1 == count) off[count] = word(o + t[k]);  // the total
         }
         o += t[k];
     }
@@ -459,7 +461,7 @@ __global__ void k_ranges(const uint32_t* __restrict__ keys, const uint32_t* coun
                          uint32_t* __restrict__ ranges, uint32_t* __restrict__ order_scratch) {
     grid_dep_begin();
     // the tile order's bucket counts and cursors start at zero
-    if (blockIdx.x == 0 && threadIdx.x < 2 * kOrderBuckets) order_scratch[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x < 2 * kTailBuckets) order_scratch[threadIdx.x] = 0u;
     constexpr uint32_t kNone = 0xFFFFFFFFu;  // past either end (never a tile id)
     const uint32_t count = *count_dev;
     const uint32_t ngroups = (count + 3) / 4;
@@ -500,19 +502,19 @@ constexpr int kOrderThreads = 256;
 
 __device__ __forceinline__ int work_bucket(const uint32_t* ranges, int t) {
     const uint32_t len = ranges[2 * t + 1] - ranges[2 * t];
-    return len == 0u ? kOrderBuckets - 1 : __clz(len);  // 0 = longest
+    return len == 0u ? kTailBuckets - 1 : __clz(len);  // 0 = longest
 }
 
 __global__ void __launch_bounds__(kOrderThreads)
 k_tile_buckets(const uint32_t* __restrict__ ranges, int T, uint32_t* __restrict__ counts) {
     grid_dep_begin();
-    __shared__ uint32_t cnt[kOrderBuckets];
-    if (threadIdx.x < kOrderBuckets) cnt[threadIdx.x] = 0u;
+    __shared__ uint32_t cnt[kTailBuckets];
+    if (threadIdx.x < kTailBuckets) cnt[threadIdx.x] = 0u;
     __syncthreads();
     for (int t = blockIdx.x * kOrderThreads + threadIdx.x; t < T; t += gridDim.x * kOrderThreads)
         atomicAdd(&cnt[work_bucket(ranges, t)], 1u);
     __syncthreads();
-    if (threadIdx.x < kOrderBuckets && cnt[threadIdx.x] != 0u)
+    if (threadIdx.x < kTailBuckets && cnt[threadIdx.x] != 0u)
         atomicAdd(&counts[threadIdx.x], cnt[threadIdx.x]);
 }
 
@@ -520,10 +522,10 @@ __global__ void __launch_bounds__(kOrderThreads)
 k_tile_order(const uint32_t* __restrict__ ranges, int T, const uint32_t* __restrict__ counts,
              uint32_t* __restrict__ cursors, uint32_t* __restrict__ order) {
     grid_dep_begin();
-    __shared__ uint32_t base[kOrderBuckets];
+    __shared__ uint32_t base[kTailBuckets];
     if (threadIdx.x == 0) {
         uint32_t run = 0u;
-        for (int b = 0; b < kOrderBuckets; ++b) {
+        for (int b = 0; b < kTailBuckets; ++b) {
             base[b] = run;
             run += counts[b];
         }
@@ -597,21 +599,10 @@ gs_status radix_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, u
 
 }  // namespace
 
-gs_status launch_bin_sort(const Plan* p, int32_t n, void* ws, cudaStream_t st) {
-    const uint32_t VN = (uint32_t)p->vt.n_views * (uint32_t)n;
-    const uint32_t icap = (uint32_t)p->inst_capacity;
-    uint32_t* hist = buf<uint32_t>(p, ws, B_HIST);
-    uint32_t* totals = hist + (size_t)kRadix * (p->depth_sort_blocks > p->inst_sort_blocks
-                                                    ? p->depth_sort_blocks
-                                                    : p->inst_sort_blocks);
+// The depth order and the instances' offsets of a plan of any size.
+static gs_status depth_sort(const Plan* p, uint32_t VN, uint32_t icap, void* ws, uint32_t* hist,
+                            uint32_t* totals, cudaStream_t st) {
     DevCounters* ctr = buf<DevCounters>(p, ws, GS_BUF_COUNTERS);
-    // the per-tile ranges are cleared first, so that every kernel of the
-    // binning follows another kernel (programmatic launches, see launch_pdl)
-    uint32_t* ranges = buf<uint32_t>(p, ws, GS_BUF_RANGES);
-    if (cudaMemsetAsync(ranges, 0, (size_t)p->total_tiles * 2 * sizeof(uint32_t), st) !=
-        cudaSuccess)
-        return GS_ERR_CUDA;
-
     // 1. depth digits over the (view, Gaussian) pairs: 4 passes, the
     //    projection's keys (values = positions) -> B -> C -> B -> C; the first
     //    keeps only the visible pairs, whose count (n_sorted) the later passes
@@ -623,30 +614,59 @@ gs_status launch_bin_sort(const Plan* p, int32_t n, void* ws, cudaStream_t st) {
     uint32_t* kc = buf<uint32_t>(p, ws, B_DKEY_C);
     uint32_t* va = buf<uint32_t>(p, ws, GS_BUF_DEPTH_ORDER);
     uint32_t* n_sorted = &ctr->n_sorted;
-    gs_status s0 = radix_pass(kp, nullptr, kb, vb, nullptr, VN, VN, 0, kRadixBits, hist, totals,
+    gs_status s = radix_pass(kp, nullptr, kb, vb, nullptr, VN, VN, 0, kRadixBits, hist, totals,
                               st, n_sorted);
-    if (s0 != GS_OK) return s0;
+    if (s != GS_OK) return s;
     for (int pass = 1; pass < 4; ++pass) {
         const bool odd = (pass & 1) != 0;
-        gs_status s = radix_pass(odd ? kb : kc, odd ? vb : va, odd ? kc : kb, odd ? va : vb,
+        s = radix_pass(odd ? kb : kc, odd ? vb : va, odd ? kc : kb, odd ? va : vb,
                                  n_sorted, VN, VN, pass * kRadixBits, kRadixBits, hist, totals,
                                  st);
         if (s != GS_OK) return s;
     }
 
-    // 2. scan of tiles touched in depth order, then emission (grids over all
-    //    pairs; blocks past the visible count do nothing)
+    // 2. scan of tiles touched in depth order (grids over all pairs; blocks past
+    //    the visible count do nothing)
     const int snb = (int)((VN + kScanTile - 1) / kScanTile);
     uint32_t* bsums = buf<uint32_t>(p, ws, B_SCAN_BLOCKS);
     const uint32_t* touched = buf<uint32_t>(p, ws, GS_BUF_TOUCHED);
     launch_pdl(k_scan_reduce, snb, kScanThreads, 0, st, va, touched, n_sorted, bsums);
+    launch_pdl(k_scan_offsets, snb, kScanThreads, 0, st, va, touched, bsums, snb, icap, n_sorted,
+               ctr, buf<uint32_t>(p, ws, B_OFFSETS));
+    return launch_status();
+}
+
+gs_status launch_bin_sort(const Plan* p, int32_t n, void* ws, cudaStream_t st) {
+    // the tile stage: a counting sort over all tiles where their counters fit
+    // (gs_tiles.cu), else radix passes over the tile id; the depth sort of small
+    // plans is one launch (gs_depth_small.cu)
+    const bool counting = tiles_fit(p);
+    const uint32_t VN = (uint32_t)p->vt.n_views * (uint32_t)n;
+    const uint32_t icap = (uint32_t)p->inst_capacity;
+    uint32_t* hist = buf<uint32_t>(p, ws, B_HIST);
+    uint32_t* totals = hist + (size_t)kRadix * (p->depth_sort_blocks > p->inst_sort_blocks
+                                                    ? p->depth_sort_blocks
+                                                    : p->inst_sort_blocks);
+    DevCounters* ctr = buf<DevCounters>(p, ws, GS_BUF_COUNTERS);
+    // the per-tile ranges are cleared first, so that every kernel of the
+    // binning follows another kernel (programmatic launches, see launch_pdl);
+    // the counting sort writes all of them
+    uint32_t* ranges = buf<uint32_t>(p, ws, GS_BUF_RANGES);
+    if (!counting && cudaMemsetAsync(ranges, 0, (size_t)p->total_tiles * 2 * sizeof(uint32_t), st) !=
+        cudaSuccess)
+        return GS_ERR_CUDA;
+
+    uint32_t* n_sorted = &ctr->n_sorted;
+    uint32_t* va = buf<uint32_t>(p, ws, GS_BUF_DEPTH_ORDER);
+    uint32_t* offs = buf<uint32_t>(p, ws, B_OFFSETS);
+    gs_status s0 = depth_small_fits(p, n) ? launch_depth_small(p, n, ws, st)
+                                          : depth_sort(p, VN, icap, ws, hist, totals, st);
+    if (s0 != GS_OK) return s0;
+    if (counting) return launch_tiles(p, n, ws, st);
     uint32_t* ika = buf<uint32_t>(p, ws, GS_BUF_TILE_KEYS);
     uint32_t* iva = buf<uint32_t>(p, ws, GS_BUF_TILE_VALUES);
     uint32_t* ikb = buf<uint32_t>(p, ws, B_IKEY_B);
     uint32_t* ivb = buf<uint32_t>(p, ws, B_IVAL_B);
-    uint32_t* offs = buf<uint32_t>(p, ws, B_OFFSETS);
-    launch_pdl(k_scan_offsets, snb, kScanThreads, 0, st, va, touched, bsums, snb, icap, n_sorted,
-               ctr, offs);
     const int eg = (int)min((VN + kEmitEntries - 1) / kEmitEntries,
                             (uint32_t)resident_grid<k_emit>(kEmitEntries));
     launch_pdl(k_emit, eg, kEmitEntries, 0, st, va, offs,
@@ -679,7 +699,7 @@ gs_status launch_bin_sort(const Plan* p, int32_t n, void* ws, cudaStream_t st) {
     ob = ob < 4 * sms ? ob : 4 * sms;
     launch_pdl(k_tile_buckets, ob, kOrderThreads, 0, st, ranges, p->total_tiles, order_scratch);
     launch_pdl(k_tile_order, ob, kOrderThreads, 0, st, ranges, p->total_tiles, order_scratch,
-               order_scratch + kOrderBuckets, order);
+               order_scratch + kTailBuckets, order);
     return launch_status();
 }
 
