@@ -29,14 +29,17 @@
 // cycles per instruction each (packed FP32 runs on the heavy pipe alone), and
 // for small launches the longest list, which one warp walks.  At 1M Gaussians,
 // 1200x680, 8x8 tiles (2.0M walked (block, Gaussian) pairs), against the kernels
-// of gs_render.cu at their best launch shape: forward 179 -> 137 us, 85 -> 51
-// warp instructions per pair; adjoint 330 -> 265 us, 138 -> 97 (the sums over the
-// block by shuffles took 43 of them, the window takes 24).  Sixteen views of a
-// 500k map: 1003 -> 645 and 1593 -> 1451 us.  200k Gaussians, 640x480, 16x16
-// tiles: 68 -> 45 and 177 -> 85 us (there the block test and the four warps per
-// tile count as well).  Tried in the adjoint and not kept: the high parts
-// rounded instead of cut (1503 us), a Newton step on 1 / (1 - alpha) (1476 us):
-// neither moved the gradients' error against 64 bits.
+// of gs_render.cu at their best launch shape: forward 182 -> 131 us, 85 -> 51
+// warp instructions per pair; adjoint 319 -> 233 us, 138 -> 84.  Sixteen views of
+// a 500k map: 1003 -> 634 and 1593 -> 1318 us.  200k Gaussians, 640x480, 16x16
+// tiles: 68 -> 38 and 177 -> 77 us (there the block test and the four warps per
+// tile count as well).  What the adjoint gained by its parts at 1M: the window's
+// sums instead of shuffles 319 -> 265 us; a window row for every slot instead of
+// for the voted ones, so that the loop has no branch, 265 -> 241; that loop
+// unrolled over the window 241 -> 233.  Tried and not kept: the high parts rounded
+// instead of cut and a Newton step on 1 / (1 - alpha) (neither moved the
+// gradients' error against 64 bits), 32 slots per stage for a sixth CTA per SM (256
+// us).  In the forward, two pairs evaluated before a vote: 137 -> 131 us.
 #include "gs_render.cuh"
 
 namespace gs {
@@ -45,6 +48,7 @@ namespace {
 constexpr int kBlock = 8;      // pixels along each side of a block
 constexpr int kWarps = 4;      // warps (blocks) per CTA
 constexpr int kChunk = 32;     // list entries staged at a time, one per lane
+constexpr int kStep = 2;       // pairs of Gaussians the forward evaluates before a vote
 constexpr unsigned kAll = 0xffffffffu;
 
 // e^p = 2^(p log2 e) by the hardware's base-2 exponential (ex2.approx.ftz): the
@@ -106,7 +110,9 @@ struct Feeder {
     template <class Pos>
     __device__ __forceinline__ void issue(const Pos& pos, int slot, int lane) {
         const int p = pos(issued);
-        tag[slot] = next;
+#pragma unroll
+        for (int k = 0; k < RING; ++k)
+            if (slot == k) tag[k] = next;
         if (p >= 0) {
             const uint32_t vg = gid_of ? __ldg(gid_of + next) : next;
             const float4* src = rec + (size_t)vg * 3;
@@ -131,7 +137,7 @@ struct Feeder {
     template <int CH, bool CULL, bool LISTPOS, class Pos>
     __device__ __forceinline__ unsigned stage(const Pos& pos, int c, int ns, int lane, float tx0,
                                               float ty0, float bx, float by, int list_base) {
-        if (RING == 1) cp_async_wait_all(); else cp_async_wait_one();
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 1) : "memory");
         __syncwarp();
         const int slot = RING == 1 ? 0 : (c & (RING - 1));
         const int p = pos(c);
@@ -146,14 +152,16 @@ struct Feeder {
             m.y = __fadd_rn(__fsub_rn(m.y, ty0), m.w);
             if (CULL) keep = meets_block(m.x, m.y, q.x, q.y, q.z, q.w, bx, by);
         }
-        const uint32_t t = RING == 1 || slot == 0 ? tag[0] : tag[RING - 1];
+        uint32_t t = tag[0];
+#pragma unroll
+        for (int k = 1; k < RING; ++k) t = slot == k ? tag[k] : t;
         const unsigned mask = __ballot_sync(kAll, keep);
         if (LISTPOS) {
             const bool fin = fabsf(col.x) < INFINITY && fabsf(col.y) < INFINITY &&
                              fabsf(col.z) < INFINITY;
             odd = (ns > 0 && odd) || __any_sync(kAll, keep && !fin);
         }
-        if (RING == 1 || slot == 0) issue(pos, 0, lane); else issue(pos, RING - 1, lane);
+        issue(pos, slot, lane);
         if (keep) {
             const int s = ns + __popc(mask & ((1u << lane) - 1u));
             float* f = reinterpret_cast<float*>(&st->par[s >> 1][0]) + (s & 1);
@@ -174,11 +182,14 @@ struct Feeder {
         }
         return mask;
     }
-    // A last pair with one slot in use: the other half never reaches a pixel.
+    // The slots from ns to the next multiple of M never reach a pixel.
+    template <int M>
     __device__ __forceinline__ void pad(int ns, int lane) {
-        if (!(ns & 1)) return;
-        if (lane < 6) reinterpret_cast<float*>(&st->par[ns >> 1][0])[2 * lane + 1] = 0.0f;
-        if (lane < 8) reinterpret_cast<float*>(&st->col[ns][0])[lane] = 0.0f;
+        const int top = (ns + M - 1) & ~(M - 1);
+        for (int s = ns; s < top; ++s) {
+            if (lane < 6) reinterpret_cast<float*>(&st->par[s >> 1][0])[2 * lane + (s & 1)] = 0.0f;
+            if (lane < 8) reinterpret_cast<float*>(&st->col[s][0])[lane] = 0.0f;
+        }
     }
     // Whether a staged Gaussian may need what most do not: it can reach alpha =
     // 0.99 (o >= 0.99), or its conic is so close to singular that rounding could
@@ -264,37 +275,44 @@ __device__ __forceinline__ void blend_one(FwdPixels<CH>& s, float2 na, const flo
 template <int CH, bool HARD, int SLOTS>
 __device__ __forceinline__ void blend_batch(FwdPixels<CH>& s, const Stage<SLOTS>& st, int ns,
                                             float2 nx0, float2 nx1, float2 ny, bool odd) {
-    for (int p = 0; 2 * p < ns; ++p) {
+    auto evaluate = [&](int p, float2& n0, float2& n1) {
         const float4 A = st.par[p][0], B = st.par[p][1], D = st.par[p][2];
         const float2 dy = add2(make_float2(A.z, A.w), ny);
         const float2 cdd = mul2(make_float2(D.x, D.y), mul2(dy, dy));
         const float2 gx = make_float2(A.x, A.y), a = make_float2(B.x, B.y),
                      nb = make_float2(B.z, B.w), no = make_float2(D.z, D.w);
-        PairAlpha e0 = pair_alpha(add2(gx, nx0), dy, cdd, a, nb, no);
-        PairAlpha e1 = pair_alpha(add2(gx, nx1), dy, cdd, a, nb, no);
-        if (HARD) {
-            e0.noG = tame(e0);
-            e1.noG = tame(e1);
+        const PairAlpha e0 = pair_alpha(add2(gx, nx0), dy, cdd, a, nb, no);
+        const PairAlpha e1 = pair_alpha(add2(gx, nx1), dy, cdd, a, nb, no);
+        n0 = HARD ? tame(e0) : e0.noG;
+        n1 = HARD ? tame(e1) : e1.noG;
+    };
+    for (int p = 0; 2 * p < ns; p += kStep) {
+        float2 n0[kStep], n1[kStep];
+        bool mine0 = false, mine1 = false;
+#pragma unroll
+        for (int k = 0; k < kStep; ++k) {
+            evaluate(p + k, n0[k], n1[k]);
+            mine0 = mine0 || fminf(n0[k].x, n0[k].y) <= -kAlphaMin;
+            mine1 = mine1 || fminf(n1[k].x, n1[k].y) <= -kAlphaMin;
         }
-        const bool hA0 = e0.noG.x <= -kAlphaMin, hA1 = e1.noG.x <= -kAlphaMin;
-        const bool hB0 = e0.noG.y <= -kAlphaMin, hB1 = e1.noG.y <= -kAlphaMin;
-        // one vote for the pair: that a pixel still accumulating blends either
-        if (!__any_sync(kAll,
-                        ((hA0 || hB0) && s.T.x > 0.0f) || ((hA1 || hB1) && s.T.y > 0.0f))) {
+        // one vote for the step: that a pixel still accumulating blends any
+        if (!__any_sync(kAll, (mine0 && s.T.x > 0.0f) || (mine1 && s.T.y > 0.0f))) {
             if (!__any_sync(kAll, fmaxf(s.T.x, s.T.y) > 0.0f)) return;
             continue;
         }
-        bool do_a = true, do_b = true;
-        if (HARD && odd) {
-            do_a = __any_sync(kAll, (hA0 && s.T.x > 0.0f) || (hA1 && s.T.y > 0.0f));
-            do_b = __any_sync(kAll, (hB0 && s.T.x > 0.0f) || (hB1 && s.T.y > 0.0f));
+#pragma unroll
+        for (int k = 0; k < kStep; ++k) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float a0 = h ? n0[k].y : n0[k].x, a1 = h ? n1[k].y : n1[k].x;
+                const bool h0 = a0 <= -kAlphaMin, h1 = a1 <= -kAlphaMin;
+                if (HARD && odd &&
+                    !__any_sync(kAll, (h0 && s.T.x > 0.0f) || (h1 && s.T.y > 0.0f)))
+                    continue;
+                blend_one<CH>(s, make_float2(h0 ? a0 : 0.0f, h1 ? a1 : 0.0f),
+                              st.col[2 * (p + k) + h], 2 * (p + k) + h);
+            }
         }
-        if (do_a)
-            blend_one<CH>(s, make_float2(hA0 ? e0.noG.x : 0.0f, hA1 ? e1.noG.x : 0.0f),
-                          st.col[2 * p], 2 * p);
-        if (do_b)
-            blend_one<CH>(s, make_float2(hB0 ? e0.noG.y : 0.0f, hB1 ? e1.noG.y : 0.0f),
-                          st.col[2 * p + 1], 2 * p + 1);
     }
 }
 
@@ -330,7 +348,7 @@ __device__ __forceinline__ void fwd_block(const ViewTable& vt, const TileCtx& tc
                                                            begin));
             ++c;
         } while (ns <= SLOTS - kChunk && c < chunks);
-        fd.pad(ns, lane);
+        fd.template pad<2 * kStep>(ns, lane);
         __syncwarp();
         s.l0 = s.l1 = -1;
         if (fd.hard(ns, lane) || fd.odd)
@@ -376,8 +394,11 @@ __device__ __forceinline__ int next_slot(uint32_t* queue) {
 }
 
 constexpr int kSlots = 2 * kChunk;
+// Chunks in flight: where the block test may leave a chunk little to do, the
+// copies of several have to overlap (two to four: 43 -> 41 us forward and 86 -> 80
+// adjoint at 200k Gaussians with 16x16 tiles).
 template <bool CULL>
-constexpr int kRing = CULL ? 2 : 1;
+constexpr int kRing = CULL ? 4 : 1;
 
 template <bool CULL>
 struct FwdShared {
@@ -386,7 +407,7 @@ struct FwdShared {
 };
 
 template <bool CULL>
-__global__ void __launch_bounds__(32 * kWarps, 8)
+__global__ void __launch_bounds__(32 * kWarps, CULL ? 5 : 8)
 k_blocks_fwd(ViewTable vt, const uint32_t* __restrict__ ranges,
              const uint32_t* __restrict__ order, const uint32_t* __restrict__ ivals,
              const uint32_t* __restrict__ gid_of, const float4* __restrict__ rec, int log2_bx,
@@ -451,11 +472,10 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1
 
 template <bool CULL, bool ABS>
 struct BwdShared {
-    float4 win[(kRows + 1) * 32];
-    float4 habs[ABS ? (kRows + 1) * 16 : 1];
+    float4 win[kRows * 32];
+    float4 habs[ABS ? kRows * 16 : 1];
     Stage<kSlots> st;
     float4 raw[kRing<CULL> * kChunk * 3];
-    int row_of[kRows + 4];  // the window rows' slots in the stage
 };
 
 // Monomials about the block's centre, as the B operand: entry [s][lane] holds
@@ -476,16 +496,16 @@ struct BwdOut {
 };
 
 // Sums the window's rows over the block and sends the gradients of the
-// Gaussians of its first `rows` rows on their way.  row_of: the rows' slots in
-// the stage.  gb: dL/dC as the B operand.
+// Gaussians of its first `rows` rows on their way.  slot0: the stage slot of row
+// 0.  gb: dL/dC as the B operand.
 template <int CH, bool ABS, int SLOTS>
 __device__ __forceinline__ void flush_window(const float4* win, const float4* habs,
-                                             const int* row_of, const Stage<SLOTS>& st,
+                                             int slot0, const Stage<SLOTS>& st,
                                              const Monomials& mono, const uint32_t (&gb)[8][2],
                                              int rows, float cx, float cy, const BwdOut& out) {
     const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
     __syncwarp();
-    const int slot = r < rows ? row_of[r] : 0;
+    const int slot = slot0 + r;
     float m[4] = {0.f, 0.f, 0.f, 0.f}, k[4] = {0.f, 0.f, 0.f, 0.f};
     float m2[4] = {0.f, 0.f, 0.f, 0.f};  // every other k-step's moments: half as long a chain of sums
 #pragma unroll
@@ -600,95 +620,63 @@ __device__ __forceinline__ void adjoint_one_block(BwdPixels<CH>& s, float2 na, f
     }
 }
 
-// The adjoint of a staged batch.  HARD: alphas are clamped and positive powers
-// skipped.
+// The adjoint of a staged batch, eight slots (a window) at a time.  Every slot
+// takes its row: nearly all reach a pixel of the block, and a row of zeros costs
+// less than finding out.  HARD: alphas are clamped and positive powers skipped.
 template <int CH, bool ABS, bool HARD, int SLOTS>
 __device__ __forceinline__ void adjoint_batch(
     BwdPixels<CH>& s, const Stage<SLOTS>& st, int ns, int from0, int from1, int checked,
-    float2 nx0, float2 nx1, float2 ny, float4* win, float4* habs, int* row_of,
-    const Monomials& mono, const uint32_t (&gb)[8][2], float cx, float cy, const BwdOut& out) {
+    float2 nx0, float2 nx1, float2 ny, float4* win, float4* habs, const Monomials& mono,
+    const uint32_t (&gb)[8][2], float cx, float cy, const BwdOut& out) {
     const int lane = threadIdx.x & 31;
-    // the lane's place in row 0 and what takes it from one row to the next
-    const int place0 = row_slot(0, lane), hop = 32, flip = 4;
-    int rows = 0;  // rows of the window in use
-    int place = place0;
-    float limA0 = -kAlphaMin, limA1 = -kAlphaMin, limB0 = -kAlphaMin, limB1 = -kAlphaMin;
-    for (int p = 0;;) {
-        const bool end = 2 * p >= ns;
-        if (rows >= kRows || (end && rows > 0)) {
-            flush_window<CH, ABS>(win, habs, row_of, st, mono, gb, min(rows, kRows), cx, cy, out);
-            rows = max(rows - kRows, 0);
-            place = place0;
-            if (rows > 0) {  // the ninth row becomes the first
-                win[place0] = win[row_slot(kRows, lane)];
-                if (ABS && lane < 16) habs[abs_slot(0, lane)] = habs[abs_slot(kRows, lane)];
-                if (lane == 0) row_of[0] = row_of[kRows];
-                place = (place0 + hop) ^ flip;
-                __syncwarp();
+    for (int g = 0; g < ns; g += kRows) {
+#pragma unroll
+        for (int k = 0; k < kRows / 2; ++k) {
+            const int slot = g + 2 * k;
+            const float4 A = st.par[slot >> 1][0], B = st.par[slot >> 1][1],
+                         D = st.par[slot >> 1][2];
+            const float2 dy = add2(make_float2(A.z, A.w), ny);
+            const float2 cdd = mul2(make_float2(D.x, D.y), mul2(dy, dy));
+            const float2 gx = make_float2(A.x, A.y), a = make_float2(B.x, B.y),
+                         nb = make_float2(B.z, B.w), no = make_float2(D.z, D.w);
+            const float2 dx0 = add2(gx, nx0), dx1 = add2(gx, nx1);
+            const PairAlpha e0 = pair_alpha(dx0, dy, cdd, a, nb, no);
+            const PairAlpha e1 = pair_alpha(dx1, dy, cdd, a, nb, no);
+            const float2 n0 = HARD ? tame(e0) : e0.noG, n1 = HARD ? tame(e1) : e1.noG;
+            bool hA0 = n0.x <= -kAlphaMin, hA1 = n1.x <= -kAlphaMin;
+            bool hB0 = n0.y <= -kAlphaMin, hB1 = n1.y <= -kAlphaMin;
+            if (slot < checked) {  // beyond some pixel's part of the list
+                hA0 = hA0 && slot >= from0;
+                hA1 = hA1 && slot >= from1;
+                hB0 = hB0 && slot + 1 >= from0;
+                hB1 = hB1 && slot + 1 >= from1;
             }
-        }
-        if (end) {
-            if (rows == 0) break;
-            continue;
-        }
-        const float4 A = st.par[p][0], B = st.par[p][1], D = st.par[p][2];
-        const float2 dy = add2(make_float2(A.z, A.w), ny);
-        const float2 cdd = mul2(make_float2(D.x, D.y), mul2(dy, dy));
-        const float2 gx = make_float2(A.x, A.y), a = make_float2(B.x, B.y),
-                     nb = make_float2(B.z, B.w), no = make_float2(D.z, D.w);
-        const float2 dx0 = add2(gx, nx0), dx1 = add2(gx, nx1);
-        const PairAlpha e0 = pair_alpha(dx0, dy, cdd, a, nb, no);
-        const PairAlpha e1 = pair_alpha(dx1, dy, cdd, a, nb, no);
-        if (p <= checked) {  // (one more than needed: puts the limits back)
-            limA0 = 2 * p >= from0 ? -kAlphaMin : -2.0f;
-            limA1 = 2 * p >= from1 ? -kAlphaMin : -2.0f;
-            limB0 = 2 * p + 1 >= from0 ? -kAlphaMin : -2.0f;
-            limB1 = 2 * p + 1 >= from1 ? -kAlphaMin : -2.0f;
-        }
-        float2 n0 = e0.noG, n1 = e1.noG;
-        if (HARD) {
-            n0 = tame(e0);
-            n1 = tame(e1);
-        }
-        const bool hA0 = n0.x <= limA0, hA1 = n1.x <= limA1;
-        const bool hB0 = n0.y <= limB0, hB1 = n1.y <= limB1;
-        const bool any_b = __any_sync(kAll, hB0 || hB1);
-        if (__any_sync(kAll, hA0 || hA1)) {
-            const float2 na = make_float2(hA0 ? n0.x : 0.0f, hA1 ? n1.x : 0.0f);
-            float2 nG = na;
-            if (HARD)
-                nG = make_float2(e0.noG.x > -kAlphaMax ? na.x : 0.0f,
-                                 e1.noG.x > -kAlphaMax ? na.y : 0.0f);
+            const float2 naA = make_float2(hA0 ? n0.x : 0.0f, hA1 ? n1.x : 0.0f);
+            const float2 naB = make_float2(hB0 ? n0.y : 0.0f, hB1 ? n1.y : 0.0f);
+            float2 nGA = naA, nGB = naB;
+            if (HARD) {
+                nGA = make_float2(e0.noG.x > -kAlphaMax ? naA.x : 0.0f,
+                                  e1.noG.x > -kAlphaMax ? naA.y : 0.0f);
+                nGB = make_float2(e0.noG.y > -kAlphaMax ? naB.x : 0.0f,
+                                  e1.noG.y > -kAlphaMax ? naB.y : 0.0f);
+            }
             adjoint_one_block<CH, ABS>(
-                s, na, nG, st.col[2 * p], win + place,
-                reinterpret_cast<float2*>(habs + abs_slot(rows, lane >> 1)) + (lane & 1), a.x,
+                s, naA, nGA, st.col[slot], win + row_slot(2 * k, lane),
+                reinterpret_cast<float2*>(habs + abs_slot(2 * k, lane >> 1)) + (lane & 1), a.x,
                 nb.x, D.x, dx0.x, dx1.x, dy.x);
-            if (lane == 0) row_of[rows] = 2 * p;
-            ++rows;  // at most eight now
-            place = (place + hop) ^ flip;
-        }
-        if (any_b) {
-            const float2 na = make_float2(hB0 ? n0.y : 0.0f, hB1 ? n1.y : 0.0f);
-            float2 nG = na;
-            if (HARD)
-                nG = make_float2(e0.noG.y > -kAlphaMax ? na.x : 0.0f,
-                                 e1.noG.y > -kAlphaMax ? na.y : 0.0f);
             adjoint_one_block<CH, ABS>(
-                s, na, nG, st.col[2 * p + 1], win + place,
-                reinterpret_cast<float2*>(habs + abs_slot(rows, lane >> 1)) + (lane & 1), a.y,
+                s, naB, nGB, st.col[slot + 1], win + row_slot(2 * k + 1, lane),
+                reinterpret_cast<float2*>(habs + abs_slot(2 * k + 1, lane >> 1)) + (lane & 1), a.y,
                 nb.y, D.y, dx0.y, dx1.y, dy.y);
-            if (lane == 0) row_of[rows] = 2 * p + 1;
-            ++rows;
-            place = (place + hop) ^ flip;
         }
-        ++p;
+        flush_window<CH, ABS>(win, habs, g, st, mono, gb, min(ns - g, kRows), cx, cy, out);
     }
 }
 
 template <int CH, bool CULL, bool ABS, int SLOTS, int RING>
 __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
                                           Feeder<SLOTS, RING>& fd, float4* win, float4* habs,
-                                          int* row_of, const Monomials& mono, float bg0, float bg1, float bg2,
+                                          const Monomials& mono, float bg0, float bg1, float bg2,
                                           const float* __restrict__ final_T,
                                           const int32_t* __restrict__ last_idx,
                                           const float* __restrict__ dL, const BwdOut& out) {
@@ -758,16 +746,16 @@ __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
             ns += __popc(mask);
             ++c;
         } while (ns <= SLOTS - kChunk && c < chunks);
-        fd.pad(ns, lane);
+        fd.template pad<kRows>(ns, lane);
         __syncwarp();
-        // pairs before this one hold slots beyond some pixel's part of the list
-        const int checked = ((int)__reduce_max_sync(kAll, (unsigned)max(from0, from1)) + 1) >> 1;
+        // slots before this one may lie beyond some pixel's part of the list
+        const int checked = (int)__reduce_max_sync(kAll, (unsigned)max(from0, from1));
         if (fd.hard(ns, lane))
             adjoint_batch<CH, ABS, true>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny, win,
-                                         habs, row_of, mono, gb, cx, cy, out);
+                                         habs, mono, gb, cx, cy, out);
         else
             adjoint_batch<CH, ABS, false>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny, win,
-                                          habs, row_of, mono, gb, cx, cy, out);
+                                          habs, mono, gb, cx, cy, out);
         __syncwarp();  // the stage has been read
     }
     cp_async_wait_all();
@@ -775,7 +763,7 @@ __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
 }
 
 template <bool CULL, bool ABS>
-__global__ void __launch_bounds__(32 * kWarps, 5)
+__global__ void __launch_bounds__(32 * kWarps, CULL ? 4 : 5)
 k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
              const uint32_t* __restrict__ order, const uint32_t* __restrict__ ivals,
              const uint32_t* __restrict__ gid_of, const float4* __restrict__ rec, int log2_bx,
@@ -805,10 +793,10 @@ k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
         const int sub = slot & ((1 << log2_blocks) - 1);
         const int bx = (sub & ((1 << log2_bx) - 1)) * kBlock, by = (sub >> log2_bx) * kBlock;
         if (tc.channels == 3)
-            bwd_block<3, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, my.row_of, mono, bg0, bg1, bg2, final_T,
+            bwd_block<3, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, mono, bg0, bg1, bg2, final_T,
                                     last_idx, dL, out);
         else
-            bwd_block<1, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, my.row_of, mono, bg0, bg1, bg2, final_T,
+            bwd_block<1, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, mono, bg0, bg1, bg2, final_T,
                                     last_idx, dL, out);
     }
 }
