@@ -5,7 +5,7 @@
 // while the GPU selects the pixels and interpolates (gs_pointcloud.cu).
 //
 // Bowyer-Watson insertion with exact predicates on integer coordinates
-// (orientation in 64-bit, in-circle in 128-bit integers) and "ghost"
+// (orientation in 64-bit, in-circle in 64- or 128-bit integers) and "ghost"
 // triangles for the outside: every hull edge (a, b) carries a triangle
 // (a, b, inf) whose "circumcircle" is the open half-plane beyond the edge
 // plus the open edge itself, so no finite super-triangle can perturb the
@@ -13,9 +13,15 @@
 // from the previous insertion, so each insertion touches O(1) triangles on
 // average.  On co-circular points the in-circle test is strict, so the
 // result is one of the valid Delaunay triangulations.
+//
+// Points of an image (coordinates below 2^14) take the in-circle test in 64-bit
+// integers, which hold it exactly; an insertion allocates nothing (its lists are
+// kept between insertions, and the cavity's fan is linked through the vertex at
+// which each boundary edge starts and ends); the curve's keys are computed once.
+// The 21754 points of a 752x480 keyframe, Grace host: 45.1 -> 8.0 ms.
 #include <algorithm>
 #include <cstdint>
-#include <unordered_map>
+#include <utility>
 #include <vector>
 
 #include "gs.h"
@@ -25,16 +31,24 @@ namespace {
 struct Tri {
     int v[3];   // counter-clockwise; -1 = the vertex at infinity (always v[2])
     int nb[3];  // neighbour across the edge opposite v[i]
+    int mark;   // insertion stamp of the cavity search
     bool alive;
 };
 
 using i64 = long long;
 using i128 = __int128;
 
+// INT: the integer type that holds the in-circle determinant exactly -- below
+// 3 |d|^2 |d|^2 for coordinate differences d: 64 bits up to 2^14, else 128.
+template <class INT>
 struct Del {
     const int32_t* xy;
     std::vector<Tri> t;
-    std::vector<int> mark;  // insertion stamp of the cavity search
+    // lists of one insertion, and by vertex (+ 1: the vertex at infinity first) the
+    // new triangle whose boundary edge starts or ends there
+    struct Edge { int a, b, outside; };
+    std::vector<int> bad, stack, starts, ends;
+    std::vector<Edge> edges;
     int stamp = 0;
 
     i64 X(int i) const { return xy[2 * i]; }
@@ -49,12 +63,12 @@ struct Del {
         const i64 adx = X(a) - X(d), ady = Y(a) - Y(d);
         const i64 bdx = X(b) - X(d), bdy = Y(b) - Y(d);
         const i64 cdx = X(c) - X(d), cdy = Y(c) - Y(d);
-        const i128 al = (i128)adx * adx + (i128)ady * ady;
-        const i128 bl = (i128)bdx * bdx + (i128)bdy * bdy;
-        const i128 cl = (i128)cdx * cdx + (i128)cdy * cdy;
-        const i128 det = (i128)adx * ((i128)bdy * cl - (i128)cdy * bl) -
-                         (i128)ady * ((i128)bdx * cl - (i128)cdx * bl) +
-                         al * ((i128)bdx * cdy - (i128)cdx * bdy);
+        const INT al = (INT)adx * adx + (INT)ady * ady;
+        const INT bl = (INT)bdx * bdx + (INT)bdy * bdy;
+        const INT cl = (INT)cdx * cdx + (INT)cdy * cdy;
+        const INT det = (INT)adx * ((INT)bdy * cl - (INT)cdy * bl) -
+                        (INT)ady * ((INT)bdx * cl - (INT)cdx * bl) +
+                        al * ((INT)bdx * cdy - (INT)cdx * bdy);
         return det > 0;
     }
 
@@ -90,12 +104,7 @@ struct Del {
     }
 
     int add(int a, int b, int c) {
-        Tri T;
-        T.v[0] = a; T.v[1] = b; T.v[2] = c;
-        T.nb[0] = T.nb[1] = T.nb[2] = -1;
-        T.alive = true;
-        t.push_back(T);
-        mark.push_back(0);
+        t.push_back(Tri{{a, b, c}, {-1, -1, -1}, 0, true});
         return (int)t.size() - 1;
     }
 
@@ -111,34 +120,35 @@ struct Del {
         const int k0 = locate(start, p);
         if (k0 < 0 || !in_circum(k0, p)) return -1;
         ++stamp;
-        std::vector<int> bad{k0}, stack{k0};
-        mark[k0] = stamp;
+        bad.assign(1, k0);
+        stack.assign(1, k0);
+        t[k0].mark = stamp;
         while (!stack.empty()) {
             const int k = stack.back();
             stack.pop_back();
             for (int i = 0; i < 3; ++i) {
                 const int q = t[k].nb[i];
-                if (q < 0 || mark[q] == stamp) continue;
+                if (q < 0 || t[q].mark == stamp) continue;
                 if (in_circum(q, p)) {
-                    mark[q] = stamp;
+                    t[q].mark = stamp;
                     bad.push_back(q);
                     stack.push_back(q);
                 }
             }
         }
         // the cavity's boundary edges, each turned into a triangle with p
-        struct Edge { int a, b, outside; };
-        std::vector<Edge> edges;
-        for (int k : bad)
+        edges.clear();
+        for (int k : bad) {
+            Tri& T = t[k];
             for (int i = 0; i < 3; ++i) {
-                const int q = t[k].nb[i];
-                if (q >= 0 && mark[q] == stamp) continue;
-                edges.push_back({t[k].v[(i + 1) % 3], t[k].v[(i + 2) % 3], q});
+                const int q = T.nb[i];
+                if (q >= 0 && t[q].mark == stamp) continue;
+                edges.push_back({T.v[(i + 1) % 3], T.v[(i + 2) % 3], q});
             }
-        for (int k : bad) t[k].alive = false;
-        std::unordered_map<long long, int> by_edge;  // directed edge (u -> v) -> new triangle
-        auto key = [](int u, int v) { return ((long long)(u + 1) << 32) ^ (unsigned)(v + 1); };
+            T.alive = false;
+        }
         int last = -1;
+        const int first = (int)t.size();
         for (const Edge& e : edges) {
             // triangle (a, b, p), with the infinite vertex rotated last
             int k;
@@ -147,68 +157,57 @@ struct Del {
             else k = add(e.a, e.b, p);
             Tri& T = t[k];
             // the outside neighbour across edge (a, b)
-            const int io = edge_index(T, e.a, e.b);
-            T.nb[io] = e.outside;
+            T.nb[edge_index(T, e.a, e.b)] = e.outside;
             if (e.outside >= 0) {
                 const int j = edge_index(t[e.outside], e.b, e.a);
                 if (j >= 0) t[e.outside].nb[j] = k;
             }
-            for (int i = 0; i < 3; ++i) by_edge[key(T.v[(i + 1) % 3], T.v[(i + 2) % 3])] = k;
+            starts[e.a + 1] = k;
+            ends[e.b + 1] = k;
             if (T.v[2] >= 0) last = k;
         }
-        // link the fan: each new edge (u -> v) meets its reverse (v -> u)
-        for (size_t s = t.size() - edges.size(); s < t.size(); ++s) {
-            Tri& T = t[s];
-            for (int i = 0; i < 3; ++i) {
-                if (T.nb[i] >= 0) continue;
-                const int u = T.v[(i + 1) % 3], v = T.v[(i + 2) % 3];
-                auto it = by_edge.find(key(v, u));
-                if (it != by_edge.end()) T.nb[i] = it->second;
-            }
+        // link the fan: the boundary is one closed walk around p, so across
+        // (b, p) lies the triangle whose edge starts at b, across (p, a) the one
+        // whose edge ends at a
+        for (size_t s = 0; s < edges.size(); ++s) {
+            Tri& T = t[first + (int)s];
+            const Edge& e = edges[s];
+            T.nb[edge_index(T, e.b, p)] = starts[e.b + 1];
+            T.nb[edge_index(T, p, e.a)] = ends[e.a + 1];
         }
         return last >= 0 ? last : (int)t.size() - 1;
     }
 };
 
-long long morton(int32_t x, int32_t y) {
-    long long m = 0;
+uint64_t morton(int32_t x, int32_t y) {
+    uint64_t m = 0;
     for (int b = 0; b < 21; ++b)
-        m |= ((long long)((x >> b) & 1) << (2 * b)) | ((long long)((y >> b) & 1) << (2 * b + 1));
+        m |= ((uint64_t)((x >> b) & 1) << (2 * b)) | ((uint64_t)((y >> b) & 1) << (2 * b + 1));
     return m;
 }
 
-}  // namespace
-
-extern "C" gs_status gs_delaunay(const int32_t* xy_host, int32_t n, int32_t* tri_host,
-                                 int32_t tri_capacity, int32_t* n_tri) {
-    if (!xy_host || !n_tri || n < 0 || tri_capacity < 0 || (tri_capacity > 0 && !tri_host))
-        return GS_ERR_INVALID;
-    *n_tri = 0;
-    for (int i = 0; i < n; ++i)
-        if (xy_host[2 * i] < 0 || xy_host[2 * i] >= (1 << 20) || xy_host[2 * i + 1] < 0 ||
-            xy_host[2 * i + 1] >= (1 << 20))
-            return GS_ERR_INVALID;
-    if (n < 3) return GS_OK;
-    std::vector<int> order(n);
-    for (int i = 0; i < n; ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        return morton(xy_host[2 * a], xy_host[2 * a + 1]) < morton(xy_host[2 * b], xy_host[2 * b + 1]);
-    });
+template <class INT>
+gs_status triangulate(const int32_t* xy_host, int32_t n, int32_t* tri_host, int32_t tri_capacity,
+                      int32_t* n_tri) {
+    // along the curve, equal points (an error) next to each other
+    std::vector<std::pair<uint64_t, int>> order(n);
+    for (int i = 0; i < n; ++i) order[i] = {morton(xy_host[2 * i], xy_host[2 * i + 1]), i};
+    std::sort(order.begin(), order.end());
     for (int i = 1; i < n; ++i)
-        if (xy_host[2 * order[i]] == xy_host[2 * order[i - 1]] &&
-            xy_host[2 * order[i] + 1] == xy_host[2 * order[i - 1] + 1])
-            return GS_ERR_INVALID;  // duplicate points
-    Del d;
+        if (order[i].first == order[i - 1].first) return GS_ERR_INVALID;  // duplicate points
+    Del<INT> d;
     d.xy = xy_host;
     d.t.reserve((size_t)6 * n + 16);
+    d.starts.assign((size_t)n + 1, -1);
+    d.ends.assign((size_t)n + 1, -1);
     // first triangle: the first point, the next one, and the first point off
     // their line (points before it are collinear and inserted afterwards)
-    const int a = order[0], b = order[1];
+    const int a = order[0].second, b = order[1].second;
     int c_pos = -1;
     for (int i = 2; i < n && c_pos < 0; ++i)
-        if (d.orient(a, b, order[i]) != 0) c_pos = i;
+        if (d.orient(a, b, order[i].second) != 0) c_pos = i;
     if (c_pos < 0) return GS_OK;  // all collinear: no triangle
-    int c = order[c_pos];
+    int c = order[c_pos].second;
     int A = a, Bv = b, C = c;
     if (d.orient(A, Bv, C) < 0) std::swap(Bv, C);
     const int t0 = d.add(A, Bv, C);
@@ -232,7 +231,7 @@ extern "C" gs_status gs_delaunay(const int32_t* xy_host, int32_t n, int32_t* tri
     int last = t0;
     for (int i = 2; i < n; ++i) {
         if (i == c_pos) continue;
-        const int r = d.insert(last, order[i]);
+        const int r = d.insert(last, order[i].second);
         if (r < 0) return GS_ERR_INVALID;
         last = r;
     }
@@ -248,4 +247,21 @@ extern "C" gs_status gs_delaunay(const int32_t* xy_host, int32_t n, int32_t* tri
     }
     *n_tri = cnt;
     return cnt > tri_capacity ? GS_ERR_CAPACITY : GS_OK;
+}
+
+}  // namespace
+
+extern "C" gs_status gs_delaunay(const int32_t* xy_host, int32_t n, int32_t* tri_host,
+                                 int32_t tri_capacity, int32_t* n_tri) {
+    if (!xy_host || !n_tri || n < 0 || tri_capacity < 0 || (tri_capacity > 0 && !tri_host))
+        return GS_ERR_INVALID;
+    *n_tri = 0;
+    int32_t most = 0;
+    for (size_t i = 0; i < 2 * (size_t)n; ++i) {
+        if (xy_host[i] < 0 || xy_host[i] >= (1 << 20)) return GS_ERR_INVALID;
+        most = std::max(most, xy_host[i]);
+    }
+    if (n < 3) return GS_OK;
+    return most < (1 << 14) ? triangulate<i64>(xy_host, n, tri_host, tri_capacity, n_tri)
+                            : triangulate<i128>(xy_host, n, tri_host, tri_capacity, n_tri);
 }
