@@ -50,14 +50,28 @@ __device__ __forceinline__ void adam4(float4& p, const float4& g, float4& m, flo
     adam1(p.w, g.w, m.w, v.w, lr.w, b1, b2, eps, ibc1, ibc2);
 }
 
+// Whether four floats' state and gradient are all zero: Gaussians no view has
+// reached yet.  The step leaves such floats as they are (m = v = 0 again, and
+// p -= lr 0 / (0 + eps) with finite factors and eps > 0), so nothing is written.
+__device__ __forceinline__ bool idle4(const float4& m, const float4& v, const float4& g) {
+    const uint32_t mv = __float_as_uint(m.x) | __float_as_uint(m.y) | __float_as_uint(m.z) |
+                        __float_as_uint(m.w) | __float_as_uint(v.x) | __float_as_uint(v.y) |
+                        __float_as_uint(v.z) | __float_as_uint(v.w);
+    const uint32_t gg = __float_as_uint(g.x) | __float_as_uint(g.y) | __float_as_uint(g.z) |
+                        __float_as_uint(g.w);
+    return (mv | (gg << 1)) == 0u;
+}
+
 __global__ void __launch_bounds__(kAdamThreads)
 k_adam(float* __restrict__ params, const float* __restrict__ grads, float* __restrict__ m,
        float* __restrict__ v, long long n, Groups groups, float b1, float b2, float eps,
-       const int32_t* __restrict__ step, int vec) {
+       const int32_t* __restrict__ step, int vec, int skip_idle) {
     __shared__ float s_bc[2];
+    grid_dep_begin();
     if (threadIdx.x == 0) adam_bias(b1, b2, *step, s_bc[0], s_bc[1]);
     __syncthreads();
     const float ibc1 = s_bc[0], ibc2 = s_bc[1];
+    const bool skip = skip_idle && isfinite(ibc1) && isfinite(ibc2);
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long done = 0;
@@ -68,12 +82,13 @@ k_adam(float* __restrict__ params, const float* __restrict__ grads, float* __res
         float4* M = reinterpret_cast<float4*>(m);
         float4* V = reinterpret_cast<float4*>(v);
         for (long long i = tid; i < n4; i += stride) {
-            float4 p0 = P[i], m0 = M[i], v0 = V[i];
+            float4 p0 = __ldcs(P + i), m0 = __ldcs(M + i), v0 = __ldcs(V + i);
             const float4 g0 = __ldcs(G + i);
+            if (skip && idle4(m0, v0, g0)) continue;
             adam4(p0, g0, m0, v0, lr4_of(groups, (uint32_t)(i << 2)), b1, b2, eps, ibc1, ibc2);
-            P[i] = p0;
-            M[i] = m0;
-            V[i] = v0;
+            __stcs(P + i, p0);
+            __stcs(M + i, m0);
+            __stcs(V + i, v0);
         }
         done = n4 << 2;
     }
@@ -194,17 +209,23 @@ k_adam_sparse(float* __restrict__ params, const float* __restrict__ grads, float
 // no tile, whose gradient the projection adjoint left unwritten): the update
 // of k_adam, bit for bit, without the loads of known zeros.  Float j of a
 // plane of S floats per Gaussian belongs to Gaussian j / S (S a compile-time
-// 1, 3 or 4, so the division is a multiply); a grid-stride loop over the
-// plane, a float4 per thread and trip (VEC) or a float.
+// 1, 3 or 4, so the division is a multiply).
+//
+// VEC (16-byte aligned buffers): float4s of the buffer, whatever the plane's own
+// alignment; the first and last floats of a plane that is not aligned (an odd
+// number of Gaussians) go one by one.
 template <int S, bool VEC>
-__device__ __forceinline__ void groups_plane(float* __restrict__ params,
-                                             const float* __restrict__ grads,
-                                             float* __restrict__ m, float* __restrict__ v,
-                                             uint32_t base, uint32_t len,
-                                             const uint8_t* __restrict__ gvis, float lr,
-                                             float b1, float b2, float eps, float ibc1,
-                                             float ibc2, uint32_t t0, uint32_t stride) {
-    auto scalar = [&](uint32_t j) {
+struct GroupsPlane {
+    float* __restrict__ params;
+    const float* __restrict__ grads;
+    float* __restrict__ m;
+    float* __restrict__ v;
+    const uint8_t* __restrict__ gvis;
+    uint32_t base, len;
+    float lr, b1, b2, eps, ibc1, ibc2;
+    bool skip;
+
+    __device__ __forceinline__ void one(uint32_t j) const {
         const uint32_t i = base + j;
         float p = params[i], mm = m[i], vv = v[i];
         const float g = gvis[(j / S) >> 5] ? grads[i] : 0.0f;
@@ -212,64 +233,109 @@ __device__ __forceinline__ void groups_plane(float* __restrict__ params,
         params[i] = p;
         m[i] = mm;
         v[i] = vv;
-    };
-    if (VEC) {
-        const uint32_t n4 = len >> 2;
-        for (uint32_t f = t0; f < n4; f += stride) {
-            const uint32_t j = 4u * f, q = (base + j) >> 2;
-            float4 p = __ldcs(reinterpret_cast<float4*>(params) + q);
-            float4 mm = __ldcs(reinterpret_cast<float4*>(m) + q);
-            float4 vv = __ldcs(reinterpret_cast<float4*>(v) + q);
-            const uint32_t ga = (j / S) >> 5, gb = ((j + 3) / S) >> 5;
-            const bool va = gvis[ga] != 0, vb = ga == gb ? va : gvis[gb] != 0;
-            float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (va && vb) {
-                g = __ldcs(reinterpret_cast<const float4*>(grads) + q);
-            } else if (va || vb) {  // the four floats straddle two groups
-                const float* gp = grads + base + j;
-                g.x = ((j / S) >> 5) == ga ? (va ? gp[0] : 0.0f) : (vb ? gp[0] : 0.0f);
-                g.y = (((j + 1) / S) >> 5) == ga ? (va ? gp[1] : 0.0f) : (vb ? gp[1] : 0.0f);
-                g.z = (((j + 2) / S) >> 5) == ga ? (va ? gp[2] : 0.0f) : (vb ? gp[2] : 0.0f);
-                g.w = vb ? gp[3] : 0.0f;
-            }
-            adam1(p.x, g.x, mm.x, vv.x, lr, b1, b2, eps, ibc1, ibc2);
-            adam1(p.y, g.y, mm.y, vv.y, lr, b1, b2, eps, ibc1, ibc2);
-            adam1(p.z, g.z, mm.z, vv.z, lr, b1, b2, eps, ibc1, ibc2);
-            adam1(p.w, g.w, mm.w, vv.w, lr, b1, b2, eps, ibc1, ibc2);
-            __stcs(reinterpret_cast<float4*>(params) + q, p);
-            __stcs(reinterpret_cast<float4*>(m) + q, mm);
-            __stcs(reinterpret_cast<float4*>(v) + q, vv);
-        }
-        if (t0 < (len & 3u)) scalar(4u * n4 + t0);  // the last len % 4 floats
-    } else {
-        for (uint32_t j = t0; j < len; j += stride) scalar(j);
     }
-}
+    // floats before the plane's first float4 boundary, and its float4s
+    __device__ __forceinline__ uint32_t head() const { return min((4u - (base & 3u)) & 3u, len); }
+    __device__ __forceinline__ uint32_t quads() const {
+        return VEC ? (len - head()) >> 2 : (len + 3u) >> 2;
+    }
+    // the floats before and behind the float4s, by eight threads
+    __device__ __forceinline__ void ends(uint32_t t) const {
+        if (!VEC) return;
+        const uint32_t h = head(), j = t < 4u ? t : h + 4u * quads() + t - 4u;
+        if (t < 4u ? j < h : j < len) one(j);
+    }
+    __device__ __forceinline__ void quad(uint32_t f) const {
+        if (!VEC) {
+            for (uint32_t j = 4u * f; j < min(4u * f + 4u, len); ++j) one(j);
+            return;
+        }
+        const uint32_t j = head() + 4u * f, q = (base + j) >> 2;
+        float4 p = __ldcs(reinterpret_cast<float4*>(params) + q);
+        float4 mm = __ldcs(reinterpret_cast<float4*>(m) + q);
+        float4 vv = __ldcs(reinterpret_cast<float4*>(v) + q);
+        const uint32_t ga = (j / S) >> 5, gb = ((j + 3) / S) >> 5;
+        const bool va = gvis[ga] != 0, vb = ga == gb ? va : gvis[gb] != 0;
+        float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (va && vb) {
+            g = __ldcs(reinterpret_cast<const float4*>(grads) + q);
+        } else if (va || vb) {  // the four floats straddle two groups
+            const float* gp = grads + base + j;
+            g.x = ((j / S) >> 5) == ga ? (va ? gp[0] : 0.0f) : (vb ? gp[0] : 0.0f);
+            g.y = (((j + 1) / S) >> 5) == ga ? (va ? gp[1] : 0.0f) : (vb ? gp[1] : 0.0f);
+            g.z = (((j + 2) / S) >> 5) == ga ? (va ? gp[2] : 0.0f) : (vb ? gp[2] : 0.0f);
+            g.w = vb ? gp[3] : 0.0f;
+        }
+        if (skip && idle4(mm, vv, g)) return;
+        adam1(p.x, g.x, mm.x, vv.x, lr, b1, b2, eps, ibc1, ibc2);
+        adam1(p.y, g.y, mm.y, vv.y, lr, b1, b2, eps, ibc1, ibc2);
+        adam1(p.z, g.z, mm.z, vv.z, lr, b1, b2, eps, ibc1, ibc2);
+        adam1(p.w, g.w, mm.w, vv.w, lr, b1, b2, eps, ibc1, ibc2);
+        __stcs(reinterpret_cast<float4*>(params) + q, p);
+        __stcs(reinterpret_cast<float4*>(m) + q, mm);
+        __stcs(reinterpret_cast<float4*>(v) + q, vv);
+    }
+};
 
-template <bool VEC>
+// FLAT: a CTA strides over pieces of 256 float4s of all planes, for maps whose
+// planes are less than a quarter of a wave of the GPU each (10k Gaussians 8.9 -> 5.9
+// us); else the grid strides over plane after plane (200k Gaussians with moments
+// everywhere: 58 us, in pieces 63).
+// HBM bounds it: 24 B per float of a zero group and 28 B of another, 12 or 16 B of
+// idle ones.  1M Gaussians of SH degree 3 of which one view has reached 45%: 254
+// -> 189 us, 350k of degree 2 (an odd number of them: planes off the 16-byte grid,
+// which went float by float) 77 -> 45 us.
+template <bool VEC, bool FLAT>
 __global__ void __launch_bounds__(kAdamThreads)
 k_adam_groups(float* __restrict__ params, const float* __restrict__ grads, float* __restrict__ m,
               float* __restrict__ v, Planes planes, uint32_t n_gauss,
               const uint8_t* __restrict__ gvis, float b1, float b2, float eps,
-              const int32_t* __restrict__ step) {
+              const int32_t* __restrict__ step, int skip_idle) {
     __shared__ float s_bc[2];
+    grid_dep_begin();
     if (threadIdx.x == 0) adam_bias(b1, b2, *step, s_bc[0], s_bc[1]);
     __syncthreads();
     const float ibc1 = s_bc[0], ibc2 = s_bc[1];
-    const uint32_t t0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    const bool skip = skip_idle && isfinite(ibc1) && isfinite(ibc2);
+    uint32_t first = 0u;  // first piece of the plane
     for (int pl = 0; pl < planes.count; ++pl) {
-        const uint32_t S = planes.stride[pl], base = planes.start[pl];
+        const uint32_t S = planes.stride[pl], base = planes.start[pl], len = S * n_gauss;
         const float lr = planes.lr[pl];
+        const uint32_t pieces = (len / 4u + kAdamThreads) / kAdamThreads;
+        auto run = [&](auto plane) {
+            const uint32_t n4 = plane.quads();
+            if (FLAT) {
+                // this CTA's pieces among [first, first + pieces)
+                const uint32_t c0 = (blockIdx.x + gridDim.x - first % gridDim.x) % gridDim.x;
+                if (c0 == 0u && threadIdx.x < 8) plane.ends(threadIdx.x);
+                for (uint32_t c = c0; c < pieces; c += gridDim.x) {
+                    const uint32_t f = c * kAdamThreads + threadIdx.x;
+                    if (f < n4) plane.quad(f);
+                }
+            } else {
+                const uint32_t t0 = blockIdx.x * blockDim.x + threadIdx.x;
+                if (t0 < 8u) plane.ends(t0);
+                for (uint32_t f = t0; f < n4; f += gridDim.x * blockDim.x) plane.quad(f);
+            }
+        };
         if (S == 3)
-            groups_plane<3, VEC>(params, grads, m, v, base, 3u * n_gauss, gvis, lr, b1, b2, eps,
-                                 ibc1, ibc2, t0, stride);
+            run(GroupsPlane<3, VEC>{params, grads, m, v, gvis, base, len, lr, b1, b2, eps, ibc1,
+                                    ibc2, skip});
         else if (S == 4)
-            groups_plane<4, VEC>(params, grads, m, v, base, 4u * n_gauss, gvis, lr, b1, b2, eps,
-                                 ibc1, ibc2, t0, stride);
+            run(GroupsPlane<4, VEC>{params, grads, m, v, gvis, base, len, lr, b1, b2, eps, ibc1,
+                                    ibc2, skip});
         else
-            groups_plane<1, VEC>(params, grads, m, v, base, n_gauss, gvis, lr, b1, b2, eps, ibc1,
-                                 ibc2, t0, stride);
+            run(GroupsPlane<1, VEC>{params, grads, m, v, gvis, base, len, lr, b1, b2, eps, ibc1,
+                                    ibc2, skip});
+        first += pieces;
     }
+}
+
+// Whether a step with these rates leaves all-zero floats as they are.
+static bool can_skip_idle(const float* lrs, int n, float eps) {
+    bool ok = eps > 0.0f;
+    for (int k = 0; k < n; ++k) ok = ok && isfinite(lrs[k]);
+    return ok;
 }
 
 __global__ void k_visibility(int n, int n_views, const uint32_t* __restrict__ touched,
@@ -331,7 +397,7 @@ gs_status launch_adam_groups(float* params, const float* grads, float* m, float*
                              float b1, float b2, float eps, int32_t* step_dev, cudaStream_t st) {
     if (n >= (int64_t(1) << 31)) return GS_ERR_UNSUPPORTED;
     Planes pl{};
-    bool vec = ((reinterpret_cast<uintptr_t>(params) | reinterpret_cast<uintptr_t>(grads) |
+    const bool vec = ((reinterpret_cast<uintptr_t>(params) | reinterpret_cast<uintptr_t>(grads) |
                  reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
     for (int k = 0; k < n_groups; ++k) {
         const int s = strides[k];
@@ -342,7 +408,6 @@ gs_status launch_adam_groups(float* params, const float* grads, float* m, float*
             pl.start[pl.count] = (uint32_t)o;
             pl.stride[pl.count] = (uint8_t)s;
             pl.lr[pl.count] = lrs[k];
-            if (o & 3) vec = false;
             ++pl.count;
         }
     }
@@ -350,9 +415,17 @@ gs_status launch_adam_groups(float* params, const float* grads, float* m, float*
     const int sms = sm_count();
     if (sms <= 0) return GS_ERR_CUDA;
     k_step_inc<<<1, 1, 0, st>>>(step_dev);
-    auto* kern = vec ? k_adam_groups<true> : k_adam_groups<false>;
-    kern<<<sms * kAdamBlocksPerSm, kAdamThreads, 0, st>>>(params, grads, m, v, pl, (uint32_t)n_gauss,
-                                               group_vis, b1, b2, eps, step_dev);
+    const bool flat = 3ll * n_gauss < (long long)sms * kAdamBlocksPerSm * kAdamThreads;
+    auto* kern = vec ? (flat ? k_adam_groups<true, true> : k_adam_groups<true, false>)
+                     : (flat ? k_adam_groups<false, true> : k_adam_groups<false, false>);
+    long long pieces = 0;
+    for (int k = 0; k < pl.count; ++k)
+        pieces += ((long long)pl.stride[k] * n_gauss / 4 + kAdamThreads) / kAdamThreads;
+    const int blocks = (int)(pieces < (long long)sms * kAdamBlocksPerSm ? pieces
+                                                                       : sms * kAdamBlocksPerSm);
+    launch_pdl(kern, blocks, kAdamThreads, 0, st, params, grads, m, v, pl, (uint32_t)n_gauss,
+               group_vis, b1, b2, eps, (const int32_t*)step_dev,
+               can_skip_idle(lrs, n_groups, eps) ? 1 : 0);
     return launch_status();
 }
 
@@ -379,8 +452,9 @@ gs_status launch_adam(float* params, const float* grads, float* m, float* v, int
     if (blocks > sms * kAdamBlocksPerSm) blocks = sms * kAdamBlocksPerSm;
     if (blocks < 1) blocks = 1;
     k_step_inc<<<1, 1, 0, st>>>(step_dev);
-    k_adam<<<blocks, kAdamThreads, 0, st>>>(params, grads, m, v, n, g, b1, b2, eps, step_dev,
-                                            aligned ? 1 : 0);
+    launch_pdl(k_adam, blocks, kAdamThreads, 0, st, params, grads, m, v, (long long)n, g, b1, b2,
+               eps, (const int32_t*)step_dev, aligned ? 1 : 0,
+               can_skip_idle(lrs, n_groups, eps) ? 1 : 0);
     return launch_status();
 }
 
