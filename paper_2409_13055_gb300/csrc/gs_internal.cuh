@@ -304,19 +304,15 @@ static __device__ __forceinline__ int tight_row_span(const TightEllipse& E, int 
     auto half = [&](float dy) {
         return __fsqrt_rn(fmaxf(0.0f, __fsub_rn(E.At, __fmul_rn(E.D, __fmul_rn(dy, dy)))));
     };
-    float xmax, xmin;
-    if (lo <= E.ds && E.ds <= hi) {
-        xmax = E.X;
-    } else {
-        xmax = fmaxf(__fmul_rn(__fadd_rn(__fmul_rn(E.negB, lo), half(lo)), E.invA),
-                     __fmul_rn(__fadd_rn(__fmul_rn(E.negB, hi), half(hi)), E.invA));
-    }
-    if (lo <= -E.ds && -E.ds <= hi) {
-        xmin = -E.X;
-    } else {
-        xmin = fminf(__fmul_rn(__fsub_rn(__fmul_rn(E.negB, lo), half(lo)), E.invA),
-                     __fmul_rn(__fsub_rn(__fmul_rn(E.negB, hi), half(hi)), E.invA));
-    }
+    // both ends' halves once, without branches: a warp's rows take both sides
+    const float bl = __fmul_rn(E.negB, lo), bh = __fmul_rn(E.negB, hi);
+    const float hl = half(lo), hh = half(hi);
+    const float right = fmaxf(__fmul_rn(__fadd_rn(bl, hl), E.invA),
+                              __fmul_rn(__fadd_rn(bh, hh), E.invA));
+    const float left = fminf(__fmul_rn(__fsub_rn(bl, hl), E.invA),
+                             __fmul_rn(__fsub_rn(bh, hh), E.invA));
+    const float xmax = lo <= E.ds && E.ds <= hi ? E.X : right;
+    const float xmin = lo <= -E.ds && -E.ds <= hi ? -E.X : left;
     // tiles [ceil((mu + xmin - T + 1) / T), floor((mu + xmax) / T)], mu as a pair
     const float it = __frcp_rn(tw);  // exact: a power of two
     float s, e;
@@ -329,6 +325,23 @@ static __device__ __forceinline__ int tight_row_span(const TightEllipse& E, int 
     *x0 = min(max(k0, rx0), rx1);
     *x1 = max(min(k1, rx1), *x0);
     return *x1 - *x0;
+}
+
+// The lanes of `among` that hold the same low `bits` (<= BITS) of d as this one
+// (every lane of the warp calls it; the answer of a lane outside `among` means
+// nothing).  One vote per bit: __match_any_sync goes through the distinct
+// values one after another, some 50 cycles of the SM a warp against 10.
+template <int BITS>
+__device__ __forceinline__ unsigned match_bits(unsigned among, uint32_t d, int bits) {
+    unsigned peers = among;
+#pragma unroll
+    for (int b = 0; b < BITS; ++b) {
+        if (b >= bits) break;
+        const bool one = (d >> b) & 1u;
+        const unsigned m = __ballot_sync(0xffffffffu, one);
+        peers &= one ? m : ~m;
+    }
+    return peers;
 }
 
 // The Gaussian's weight at a pixel, evaluated identically by the forward and
