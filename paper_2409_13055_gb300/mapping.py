@@ -556,7 +556,8 @@ class GSRender(torch.autograd.Function):
                                "workspace no longer holds this render's projection (use a "
                                "recompute rasteriser, recompute=True, or one rasteriser per "
                                "pending render)")
-        g = [torch.zeros_like(t) for t in (means, log_scales, quats, opacity_logits, sh)]
+        # (every element is written: the adjoint overwrites, zeros included)
+        g = [torch.empty_like(t) for t in (means, log_scales, quats, opacity_logits, sh)]
         grads = B.gs_map_grad(*[t.data_ptr() for t in g])
         rast.render_bwd(gmap, grads, dL=dimages.contiguous(), final_T=final_T, last_idx=last_idx)
         return (*g, None, None)
@@ -571,7 +572,7 @@ class L1SSIMLoss(torch.autograd.Function):
     @staticmethod
     def forward(ctx, images, targets, rast: Rasterizer, lam):
         images = images.contiguous()
-        loss = torch.zeros(1, dtype=torch.float32, device=images.device)
+        loss = torch.empty(1, dtype=torch.float32, device=images.device)
         dL = torch.empty_like(images)
         B.gs_loss_l1_ssim(rast.plan, images, targets, lam, 1.0 / len(rast.views), loss, dL,
                           rast.ws)
