@@ -285,7 +285,17 @@ def run_reference(args, ws, rank):
 # ----------------------------------------------------------------------------
 def tile_passes(total_tiles):
     bits = max(1, math.ceil(math.log2(max(2, total_tiles))))
-    return (bits + 7) // 8
+    return (bits + 9) // 10
+
+
+def bin_launches(rast, n):
+    """Kernels of one binning, as the library picks its routes: the depth sort in
+    one launch up to 131072 pairs, else three radix passes and two scans; the tile
+    stage as a counting sort in three, else emission, radix passes over the tile
+    id, ranges and the order in two."""
+    depth = 1 if n * rast.views_per_pass <= 131072 else 3 * 3 + 2
+    counting = rast.instance_capacity <= 1 << 20 and rast.total_tiles <= 24000
+    return depth + (3 if counting else 1 + 3 * tile_passes(rast.total_tiles) + 3)
 
 
 def run_batched(args, ws):
@@ -772,7 +782,7 @@ def run_gpu(args, ws, rank, local):
     K_sh = (gm.degree + 1) ** 2
     algo_bytes = dict(
         project=n * (4 * (11 + 3 * K_sh)) + n * 72,
-        bin_sort=n * 4 * 16 + n * 12 + instances * 8 + tile_passes(rast.total_tiles) * instances * 16
+        bin_sort=n * 4 * 12 + n * 12 + instances * 8 + tile_passes(rast.total_tiles) * instances * 16
         + instances * 4 + rast.total_tiles * 8,
         loss_l1_ssim=rast.total_values * 44,
         # parameters read (44 + 12K B), gradients written (same), screen-space
@@ -807,11 +817,11 @@ def run_gpu(args, ws, rank, local):
                     peak_source="%d SMs (device) x 128 FP32 lanes x 2 x sm_max_mhz (%s)" % (
                         peaks["sms"], peaks["source"]))
 
-    # project 1, bin_sort 18 + 3 per tile-id pass, render_fwd 1, loss 2,
+    # project 1, bin_sort, render_fwd 1, loss 2,
     # render_bwd 1, then the projection adjoint (one kernel for one view) +
     # step counter + adam (+ the visibility kernel for sparse), or step
     # counter + the fused adjoint kernel
-    launches_per_step = 1 + (18 + 3 * tile_passes(rast.total_tiles)) + 1 + 2 + 1 + \
+    launches_per_step = 1 + bin_launches(rast, n) + 1 + 2 + 1 + \
         {"fused": 2, "separate": 3, "sparse": 4}[args.adam]
 
     out = dict(metric=METRIC, value=value, unit="iters/s", n_gpus=ws, steps=K, warmup=args.warmup,

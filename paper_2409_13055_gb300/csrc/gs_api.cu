@@ -114,13 +114,16 @@ extern "C" gs_status gs_plan_init(gs_plan* plan, const gs_config* cfg, int32_t n
     int bits = 0;
     while ((int64_t(1) << bits) < bin_tiles) ++bits;
     p->tile_bits = bits < 1 ? 1 : bits;
-    p->tile_passes = (p->tile_bits + kRadixBits - 1) / kRadixBits;
+    p->tile_passes = (p->tile_bits + kTileDigitBits - 1) / kTileDigitBits;
 
     // (view, Gaussian) pairs the workspace holds: all views', or one view's
     // in a recompute plan (views then go through it one pass at a time)
     const int64_t VN = (int64_t)p->ws_views * n_capacity;
-    p->depth_sort_blocks = (int32_t)((VN + kSortTile - 1) / kSortTile);
-    p->inst_sort_blocks = (int32_t)((instance_capacity + kSortTile - 1) / kSortTile);
+    {
+        const int64_t depth = sort_blocks(VN) << kDepthBits;
+        const int64_t inst = sort_blocks(instance_capacity) << kTileDigitBits;
+        p->hist_words = depth > inst ? depth : inst;
+    }
     p->scan_blocks = (int32_t)((VN + kScanTile - 1) / kScanTile);
     // loss: 32x16 output tiles per channel plane
     int64_t lb = 0;
@@ -149,11 +152,7 @@ extern "C" gs_status gs_plan_init(gs_plan* plan, const gs_config* cfg, int32_t n
     len[B_DVAL_B] = (size_t)VN * sizeof(uint32_t);
     len[B_DKEY_C] = (size_t)VN * sizeof(uint32_t);
     len[B_SCAN_BLOCKS] = (size_t)(p->scan_blocks + 1) * sizeof(uint32_t) * 2;
-    {
-        int mb = p->depth_sort_blocks > p->inst_sort_blocks ? p->depth_sort_blocks
-                                                             : p->inst_sort_blocks;
-        len[B_HIST] = ((size_t)kRadix * mb + kRadix) * sizeof(uint32_t);
-    }
+    len[B_HIST] = ((size_t)p->hist_words + (1u << kDepthBits)) * sizeof(uint32_t);
     len[B_IKEY_B] = (size_t)instance_capacity * sizeof(uint32_t);
     len[B_IVAL_B] = (size_t)instance_capacity * sizeof(uint32_t);
     len[B_LOSS_MAPS] = (size_t)values * 3 * sizeof(float);
@@ -248,7 +247,7 @@ extern "C" gs_status gs_plan_view_pass(const gs_plan* plan, int32_t k, gs_plan* 
     int bits = 0;
     while ((int64_t(1) << bits) < q->total_tiles) ++bits;
     q->tile_bits = bits < 1 ? 1 : bits;
-    q->tile_passes = (q->tile_bits + kRadixBits - 1) / kRadixBits;
+    q->tile_passes = (q->tile_bits + kTileDigitBits - 1) / kTileDigitBits;
     q->loss_blocks = blocks;
     return GS_OK;
 }

@@ -19,11 +19,22 @@ constexpr int kOrderSub = 8;  // tile-order buckets per octave of the list lengt
 constexpr int kOrderBuckets = 33 * kOrderSub;
 constexpr int kCountRows = 160;       // CTAs of the counting tile sort at most
 constexpr int kCountTiles = 24000;  // tiles it takes at most (their counters are shared memory)
-constexpr int kRadixBits = 8;
-constexpr int kRadix = 1 << kRadixBits;
+// The radix passes (gs_sort.cu): digits of at most kTileDigitBits bits over the
+// instances and kDepthBits over the pairs; blocks of 1024 keys below kSortLarge
+// keys, of 2048 from there on.
+constexpr int kTileDigitBits = 10;
+constexpr int kDepthBits = 11;
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 4;
-constexpr int kSortTile = kSortThreads * kSortItems;  // elements per sort block
+constexpr int kSortItems = 4, kSortItemsLarge = 8;
+constexpr int64_t kSortLarge = int64_t(1) << 20;
+// Blocks of any number of keys up to `most` (fewer keys can take more blocks).
+inline int64_t sort_blocks(int64_t most) {
+    const int64_t small = (most + kSortThreads * kSortItems - 1) / (kSortThreads * kSortItems);
+    const int64_t large = (most + kSortThreads * kSortItemsLarge - 1) / (kSortThreads * kSortItemsLarge);
+    if (most < kSortLarge) return small;
+    const int64_t edge = kSortLarge / (kSortThreads * kSortItems);
+    return large > edge ? large : edge;
+}
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;  // elements per scan block
@@ -85,7 +96,8 @@ struct Plan {
     int64_t inst_capacity;
     int32_t total_tiles, tile_bits, tile_passes;
     int64_t total_pixels, total_values;
-    int32_t depth_sort_blocks, inst_sort_blocks, scan_blocks, loss_blocks;
+    int32_t scan_blocks, loss_blocks;
+    int64_t hist_words;  // of B_HIST, before the digits' totals
     uint32_t span_pool_rows;  // capacity of B_SPAN_POOL (tight plans)
     // Recompute plans (gs_config.recompute = views per pass): the workspace
     // holds the projection and binning of ws_views views; the plan itself
@@ -110,6 +122,7 @@ struct DevCounters {
     uint32_t vn;                   // depth-order entries (visible pairs) of the last gs_bin_sort
     uint32_t n_sorted;             // visible pairs kept by the first depth pass
     uint32_t span_pool_used;       // rows of B_SPAN_POOL taken by the last gs_project
+    uint32_t max_key;              // largest depth key of its visible pairs
 };
 
 static_assert(offsetof(DevCounters, status) == 0, "gs_project keeps the leading status word");
@@ -327,16 +340,17 @@ static __device__ __forceinline__ int tight_row_span(const TightEllipse& E, int 
     return *x1 - *x0;
 }
 
-// The lanes of `among` that hold the same low `bits` (<= BITS) of d as this one
+// The lanes of `among` that hold the same d (< 2^bits, bits <= BITS) as this one
 // (every lane of the warp calls it; the answer of a lane outside `among` means
-// nothing).  One vote per bit: __match_any_sync goes through the distinct
-// values one after another, some 50 cycles of the SM a warp against 10.
+// nothing).  One vote per bit, whatever the number of distinct values.
 template <int BITS>
 __device__ __forceinline__ unsigned match_bits(unsigned among, uint32_t d, int bits) {
     unsigned peers = among;
 #pragma unroll
     for (int b = 0; b < BITS; ++b) {
-        if (b >= bits) break;
+        // (a bit past the width is zero in every lane: tested from the eighth on,
+        // two at a time)
+        if (b >= 7 && b % 2 == 1 && b >= bits) break;
         const bool one = (d >> b) & 1u;
         const unsigned m = __ballot_sync(0xffffffffu, one);
         peers &= one ? m : ~m;

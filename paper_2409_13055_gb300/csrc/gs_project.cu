@@ -393,6 +393,8 @@ k_project(const float* __restrict__ means, const float* __restrict__ log_scales,
           uint32_t* __restrict__ spans, uint32_t* __restrict__ pool, uint32_t pool_rows) {
     __shared__ Cam cams[kViewsPerThread];
     __shared__ Reach reach[kViewsPerThread];
+    __shared__ uint32_t known;
+    if (threadIdx.x == 64) known = *(volatile uint32_t*)&counters->max_key;
     const int v0 = blockIdx.y * kViewsPerThread;
     const int nv = min(kViewsPerThread, vt.n_views - v0);
     if (threadIdx.x < nv) load_cam(views[v0 + threadIdx.x], cams[threadIdx.x]);
@@ -401,7 +403,9 @@ k_project(const float* __restrict__ means, const float* __restrict__ log_scales,
                    near_z, reach[threadIdx.x - 32]);
     __syncthreads();
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned warp = __ballot_sync(0xffffffffu, g < n);
     if (g >= n) return;
+    uint32_t most = 0u;  // largest depth key
     // the map is streamed once per projection: evict-first loads, so that
     // the records written here stay in the L2 for the render kernels
     const float mean[3] = {__ldcs(means + 3 * g), __ldcs(means + 3 * g + 1),
@@ -500,12 +504,17 @@ k_project(const float* __restrict__ means, const float* __restrict__ log_scales,
         r[2] = make_float4(col[0], col[1], col[2], p.xc[2]);
         touched[vg] = area;
         dkey[vg] = __float_as_uint(p.xc[2]);
+        most = max(most, __float_as_uint(p.xc[2]));
         radius_out[vg] = p.radius;
         uint2 rc;
         rc.x = (uint32_t)p.rect[0] | ((uint32_t)p.rect[1] << 16);
         rc.y = (uint32_t)p.rect[2] | ((uint32_t)p.rect[3] << 16);
         reinterpret_cast<uint2*>(rect_out)[vg] = rc;
     }
+    // the depth sort's digits are those of the largest key; few warps are above
+    // what the word held when their CTA started
+    most = __reduce_max_sync(warp, most);
+    if ((threadIdx.x & 31) == 0 && most > known) atomicMax(&counters->max_key, most);
 }
 
 // Whether any Gaussian of this warp's group of 32 touches a tile in any view

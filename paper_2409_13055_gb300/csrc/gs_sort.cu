@@ -2,15 +2,20 @@
 //
 // The order the rasteriser needs (paper Sec. II: depth sorting; Sec. III-B:
 // tile-based rasterisation) is that of the key (tile, depth, view*n+index).
-// It is produced as one stable LSD radix sort whose low digits -- the 32 bits
-// of the FP32 depth -- are sorted once per (view, Gaussian) *before* the
-// instances are emitted (all instances of a Gaussian share its depth), and
-// whose high digits -- the global tile id -- are sorted over the emitted
-// instances.  Emission walks the depth order, so the instance array enters
+// It is produced as one stable LSD radix sort whose low digits -- the bits of
+// the FP32 depth above the near plane's -- are sorted once per (view, Gaussian)
+// *before* the instances are emitted (all instances of a Gaussian share its
+// depth), and whose high digits -- the global tile id -- are sorted over the
+// emitted instances.  Emission walks the depth order, so the instance array enters
 // the tile passes already in (depth, view, index) order and stability keeps
 // it.  Per pass: a per-block digit histogram, a per-digit scan over blocks and
-// a stable block-local ranking with warp match + per-warp counters, scattered
-// to the digit's global offset.  The first depth pass drops the (view,
+// a stable block-local ranking by warp votes + per-warp counters, scattered
+// to the digit's global offset.  What bounds a pass is the latency of those
+// steps within a block (issue slots half busy, a quarter of the bandwidth), so
+// there are few of them: three over the depth, digits of up to ten bits over the
+// tile id.  Whole binning with four 8-bit depth passes and 8-bit tile digits ->
+// now: 13.8M instances of 16 views 735 -> 590 us, 3.3M of two views of 2M 280 ->
+// 260, 3.1M of one of 1M 159 -> 148, 444k of 350k pairs 65 -> 60.  The first depth pass drops the (view,
 // Gaussian) pairs the projection culled (key 0xFFFFFFFF, no tile): the later
 // passes, the scan and the emission run over the visible pairs only, whose
 // count stays on the device like the instance count.  No kernel waits on
@@ -62,96 +67,187 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* w
     return r;
 }
 
-// Radix passes over blocks of ITEMS keys per thread (TILE = 256 * ITEMS keys
-// per block).
+// Digit of a radix pass: `width` bits from `shift` of (key - sub), or, for the
+// depth sort (ctr given), its pass `shift` of kDepthPasses: the bits that the
+// largest key less the smallest possible one (sub = the near plane's) has,
+// split evenly -- eight or nine bits a pass in place of four passes of eight.
+// At most kDigits values: 31 bits, the most a positive float has, in three.
+struct Digit {
+    const DevCounters* ctr;
+    uint32_t sub;
+    int shift, width;
+};
+constexpr int kDepthPasses = 3;
+constexpr int kDigits = 1 << kDepthBits;
+static_assert(kDepthPasses * kDepthBits >= 31, "every positive float");
+
+struct DigitOf {
+    uint32_t sub, mask;
+    int shift, width;
+    __device__ __forceinline__ explicit DigitOf(const Digit& d)
+        : sub(d.sub), shift(d.shift), width(d.width) {
+        if (d.ctr) {
+            const uint32_t most = d.ctr->max_key;  // 0: no visible pair
+            const int bits = 32 - __clz((most > sub ? most - sub : 0u) | 1u);
+            width = min((bits + kDepthPasses - 1) / kDepthPasses, kDepthBits);
+            shift = d.shift * width;
+        }
+        mask = (1u << width) - 1u;
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t key) const {
+        return ((key - sub) >> shift) & mask;
+    }
+};
+
+// Radix passes over blocks of ITEMS keys per thread (TILE = kSortThreads *
+// ITEMS keys per block).  hist is [digit][block], a row of nb words per digit.
 template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads)
 k_radix_hist(const uint32_t* __restrict__ keys, const uint32_t* count_dev, uint32_t count_host,
-             uint32_t cap, int shift, uint32_t mask, int nb, int drop,
-             uint32_t* __restrict__ hist) {
+             uint32_t cap, Digit dg, int nb, int drop, uint32_t* __restrict__ hist) {
     grid_dep_begin();
     constexpr int TILE = kSortThreads * ITEMS;
-    __shared__ uint32_t h[kRadix];
+    extern __shared__ uint32_t h[];
+    const DigitOf digit(dg);
     const uint32_t count = min(active_count(count_dev, count_host), cap);
     // a grid of resident CTAs striding over the sort blocks of the active keys
     for (uint32_t blk = blockIdx.x; blk * (uint32_t)TILE < count; blk += gridDim.x) {
         const uint32_t start = blk * (uint32_t)TILE;
-        h[threadIdx.x] = 0u;
+        constexpr int V = ITEMS >= 4 ? ITEMS / 4 : 1;
+        constexpr uint32_t W = ITEMS >= 4 ? 4u : (uint32_t)ITEMS;  // keys per load
+        uint4 k[V];
+#pragma unroll
+        for (int r = 0; r < V; ++r) {
+            const uint32_t i = start + W * (r * kSortThreads + threadIdx.x);
+            if (i + W <= count) {
+                if (W == 4) {
+                    k[r] = *reinterpret_cast<const uint4*>(keys + i);
+                } else {
+                    const uint2 x = *reinterpret_cast<const uint2*>(keys + i);
+                    k[r] = make_uint4(x.x, x.y, 0u, 0u);
+                }
+            }
+        }
+        for (int d = threadIdx.x; d <= (int)digit.mask; d += kSortThreads) h[d] = 0u;
         __syncthreads();
-        const uint32_t end = min(start + (uint32_t)TILE, count);
-        for (uint32_t i = start + threadIdx.x; i < end; i += kSortThreads) {
-            const uint32_t k = keys[i];
-            if (!(drop && k == kCulledKey)) atomicAdd(&h[(k >> shift) & mask], 1u);
+        auto add = [&](uint32_t key) {
+            if (!(drop && key == kCulledKey)) atomicAdd(&h[digit(key)], 1u);
+        };
+#pragma unroll
+        for (int r = 0; r < V; ++r) {
+            const uint32_t i = start + W * (r * kSortThreads + threadIdx.x);
+            if (i + W <= count) {
+                add(k[r].x);
+                add(k[r].y);
+                if (W == 4) {
+                    add(k[r].z);
+                    add(k[r].w);
+                }
+            } else {
+                for (uint32_t j = i; j < count; ++j) add(keys[j]);
+            }
         }
         __syncthreads();
-        hist[(size_t)threadIdx.x * nb + blk] = h[threadIdx.x];
+        for (int d = threadIdx.x; d <= (int)digit.mask; d += kSortThreads)
+            hist[(size_t)d * nb + blk] = h[d];
+        __syncthreads();
     }
 }
 
-// One block per digit: exclusive scan of the digit's per-block counts (in
-// place) and the digit total.
+// A CTA per digit (striding): exclusive scan of the digit's per-block counts
+// (in place) and the digit total.
 template <int ITEMS>
-__global__ void __launch_bounds__(kSortThreads)
+__global__ void __launch_bounds__(kScanThreads)
 k_radix_scan(uint32_t* __restrict__ hist, const uint32_t* count_dev, uint32_t count_host,
-             uint32_t cap, int nb, uint32_t* __restrict__ totals) {
+             uint32_t cap, Digit dg, int nb, uint32_t* __restrict__ totals) {
     grid_dep_begin();
     constexpr int TILE = kSortThreads * ITEMS;
     __shared__ uint32_t wt[33];
+    const DigitOf digit(dg);
     const uint32_t count = min(active_count(count_dev, count_host), cap);
     const int active = (int)((count + TILE - 1) / TILE);
-    uint32_t* row = hist + (size_t)blockIdx.x * nb;
-    uint32_t carry = 0;
-    for (int base = 0; base < active; base += kSortThreads * 4) {
-        uint32_t v[4], s = 0;
-        for (int k = 0; k < 4; ++k) {
-            int i = base + threadIdx.x * 4 + k;
-            v[k] = i < active ? row[i] : 0u;
-            s += v[k];
+    for (int d = blockIdx.x; d <= (int)digit.mask; d += gridDim.x) {
+        uint32_t* row = hist + (size_t)d * nb;
+        uint32_t carry = 0;
+        for (int base = 0; base < active; base += kScanThreads * 4) {
+            uint32_t v[4], s = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                int i = base + threadIdx.x * 4 + k;
+                v[k] = i < active ? row[i] : 0u;
+                s += v[k];
+            }
+            uint32_t tot;
+            uint32_t ex = block_exclusive_scan(s, wt, tot);
+            uint32_t run = carry + ex;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                int i = base + threadIdx.x * 4 + k;
+                if (i < active) row[i] = run;
+                run += v[k];
+            }
+            carry += tot;
         }
-        uint32_t tot;
-        uint32_t ex = block_exclusive_scan(s, wt, tot);
-        uint32_t run = carry + ex;
-        for (int k = 0; k < 4; ++k) {
-            int i = base + threadIdx.x * 4 + k;
-            if (i < active) row[i] = run;
-            run += v[k];
-        }
-        carry += tot;
+        if (threadIdx.x == 0) totals[d] = carry;
     }
-    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
 // Stable scatter of one block of keys: each key's rank among the block's keys
-// of its digit comes from per-warp match_any ranking; the block is first
+// of its digit comes from per-warp ranking by votes (match_bits); the block is first
 // reordered by digit in shared memory, so the global writes of each digit's
 // run are consecutive addresses (coalesced) instead of one scattered word per
 // key.  With drop, culled keys are neither ranked nor written, and block 0
 // stores the number of keys the pass keeps in *kept_out.  Without vals_in
-// the value of key i is i.
+// the value of key i is i; without keys_out only the values are written.
+// Shared memory: a word per digit, and either the warps' 16-bit counters of the
+// digits or the reordered block (so that 2048 digits leave four CTAs an SM).
+// 13.8M keys by nine bits 105-116 us, by six bits 85; CTAs of 512 threads and
+// 4096 keys 120-130.
+__host__ __device__ constexpr size_t scatter_smem(int digits, int items) {
+    const size_t counters = (size_t)digits * 2 * kWarps, block = (size_t)kSortThreads * items * 8;
+    return (size_t)digits * 4 + (counters > block ? counters : block);
+}
+
 template <int ITEMS>
-__global__ void __launch_bounds__(kSortThreads)
+__global__ void __launch_bounds__(kSortThreads, 4)
 k_radix_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
                 uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out,
-                const uint32_t* count_dev, uint32_t count_host, uint32_t cap, int shift,
-                uint32_t mask, int nb,
+                const uint32_t* count_dev, uint32_t count_host, uint32_t cap, Digit dg, int nb,
                 const uint32_t* __restrict__ hist, const uint32_t* __restrict__ totals, int drop,
                 uint32_t* __restrict__ kept_out) {
     grid_dep_begin();
     constexpr int TILE = kSortThreads * ITEMS;
+    static_assert(TILE < 65536 && kDigits <= 65536, "places and digits are 16 bits");
     constexpr int kWarpItems = TILE / kWarps;  // consecutive keys per warp
-    __shared__ uint32_t base[kRadix];          // global start of the digit's run of this block
-    __shared__ uint32_t local[kRadix];         // start of the digit's run inside the block
-    __shared__ uint32_t wcnt[kWarps][kRadix];
+    extern __shared__ uint32_t dyn[];
     __shared__ uint32_t wt[33];
-    __shared__ uint32_t skey[TILE], sval[TILE];
+    const DigitOf digit(dg);
+    const int D = (int)digit.mask + 1;
+    uint32_t* const delta = dyn;  // a digit's place in the output less that in the block
+    uint32_t* const pairs = delta + D;  // the counters: [warp][two digits]
+    uint32_t* const skey = delta + D;
+    uint32_t* const sval = skey + TILE;
     const uint32_t count = min(active_count(count_dev, count_host), cap);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    uint16_t* const mine = reinterpret_cast<uint16_t*>(pairs + w * (D / 2));
+    // a thread's digits are consecutive pairs: first, first + 1, ...
+    const int per = (D / 2 + kSortThreads - 1) / kSortThreads;
+    const int first = min(tid * per, D / 2), last = min(first + per, D / 2);
+    // start of the thread's first digit in the output
+    uint32_t digit0;
+    {
+        uint32_t s = 0u, tot;
+        for (int j = 2 * first; j < 2 * last; ++j) s += totals[j];
+        digit0 = block_exclusive_scan(s, wt, tot);
+        if (kept_out && blockIdx.x == 0 && tid == 0) *kept_out = tot;  // keys of all digits
+    }
     // a grid of resident CTAs striding over the sort blocks of the active keys
     for (uint32_t blk = blockIdx.x; blk * (uint32_t)TILE < count; blk += gridDim.x) {
         const uint32_t start = blk * (uint32_t)TILE;
         // the block's keys and values are loaded first, so that their latency
-        // overlaps the loads and the scan of the digit offsets below
-        uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
+        // overlaps the loads of the digit offsets below
+        uint32_t key[ITEMS], val[ITEMS];
+        uint32_t rank[ITEMS];  // digit << 16 | rank within the warp, then place in the block
         const uint32_t wstart = start + (uint32_t)w * kWarpItems;
 #pragma unroll
         for (int r = 0; r < ITEMS; ++r) {
@@ -161,60 +257,81 @@ k_radix_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
             val[r] = in ? (vals_in ? vals_in[i] : i) : 0u;
         }
         {
-            uint32_t tot;
-            uint32_t ex = block_exclusive_scan(totals[tid], wt, tot);
-            base[tid] = ex + hist[(size_t)tid * nb + blk];
-            if (kept_out && blk == 0 && tid == 0) *kept_out = tot;  // keys of all digits
+            uint32_t run = digit0;
+            for (int j = 2 * first; j < 2 * last; ++j) {
+                delta[j] = run + hist[(size_t)j * nb + blk];
+                run += totals[j];
+            }
         }
-#pragma unroll
-        for (int k = 0; k < kWarps; ++k) wcnt[k][tid] = 0u;
+        for (int i = tid; i < kWarps * D / 2; i += kSortThreads) pairs[i] = 0u;
         __syncthreads();
 
         const uint32_t lt = (1u << lane) - 1u;
+        unsigned kept = 0u;  // items of this lane that are written
 #pragma unroll
         for (int r = 0; r < ITEMS; ++r) {
             const uint32_t i = wstart + (uint32_t)r * 32u + lane;
-            const bool in = i < count;
-            const bool ok = in && !(drop && key[r] == kCulledKey);
-            const uint32_t d = ok ? ((key[r] >> shift) & mask) : 0x10000u;
-            const uint32_t peers = __match_any_sync(0xffffffffu, d);
+            const bool ok = i < count && !(drop && key[r] == kCulledKey);
+            const uint32_t d = digit(key[r]);
+            const uint32_t peers =
+                match_bits<kDepthBits>(__ballot_sync(0xffffffffu, ok), d, digit.width);
             uint32_t rk = 0u;
-            if (ok) rk = wcnt[w][d] + __popc(peers & lt);
+            if (ok) {
+                rk = mine[d];
+                kept |= 1u << r;
+            }
             __syncwarp();
-            if (ok && (__ffs(peers) - 1) == lane) wcnt[w][d] += __popc(peers);
+            if (ok && (peers & lt) == 0u) mine[d] = (uint16_t)(rk + __popc(peers));
             __syncwarp();
-            rank[r] = rk;
+            rank[r] = (d << 16) | (rk + __popc(peers & lt));
         }
         __syncthreads();
-        uint32_t digit_count = 0u;
+        // counts of the warps -> places in the block, two digits at a time
+        uint32_t sum = 0u;
+        for (int j = first; j < last; ++j) {
+            uint32_t two = 0u;
 #pragma unroll
-        for (int k = 0; k < kWarps; ++k) {
-            const uint32_t c = wcnt[k][tid];
-            wcnt[k][tid] = digit_count;
-            digit_count += c;
+            for (int k = 0; k < kWarps; ++k) two += pairs[k * (D / 2) + j];
+            sum += (two & 0xFFFFu) + (two >> 16);
         }
         uint32_t n_kept;  // keys of this block that are written (all of them without drop)
-        local[tid] = block_exclusive_scan(digit_count, wt, n_kept);
+        uint32_t local = block_exclusive_scan(sum, wt, n_kept);
+        for (int j = first; j < last; ++j) {
+            uint32_t c[kWarps], two = 0u;
+#pragma unroll
+            for (int k = 0; k < kWarps; ++k) {
+                c[k] = pairs[k * (D / 2) + j];
+                two += c[k];
+            }
+            const uint32_t second = local + (two & 0xFFFFu);
+            delta[2 * j] -= local;
+            delta[2 * j + 1] -= second;
+            uint32_t at = local | (second << 16);
+#pragma unroll
+            for (int k = 0; k < kWarps; ++k) {
+                pairs[k * (D / 2) + j] = at;
+                at += c[k];
+            }
+            local = second + (two >> 16);
+        }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < ITEMS; ++r) {
-            const uint32_t i = wstart + (uint32_t)r * 32u + lane;
-            if (i < count && !(drop && key[r] == kCulledKey)) {
-                const uint32_t d = (key[r] >> shift) & mask;
-                const uint32_t s = local[d] + wcnt[w][d] + rank[r];
-                skey[s] = key[r];
-                sval[s] = val[r];
+        for (int r = 0; r < ITEMS; ++r) rank[r] = mine[rank[r] >> 16] + (rank[r] & 0xFFFFu);
+        __syncthreads();  // the counters' memory takes the block
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r)
+            if ((kept >> r) & 1u) {
+                skey[rank[r]] = key[r];
+                sval[rank[r]] = val[r];
             }
-        }
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < ITEMS; ++r) {
             const int s = r * kSortThreads + tid;
             if ((uint32_t)s < n_kept) {
                 const uint32_t k = skey[s];
-                const uint32_t d = (k >> shift) & mask;
-                const uint32_t pos = base[d] + ((uint32_t)s - local[d]);
-                keys_out[pos] = k;
+                const uint32_t pos = delta[digit(k)] + (uint32_t)s;
+                if (keys_out) keys_out[pos] = k;
                 vals_out[pos] = sval[s];
             }
         }
@@ -223,18 +340,29 @@ k_radix_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
 }
 
 // Sum of tiles touched over each scan block, in depth order (the first
-// *count_dev entries of order: the visible pairs).
+// *count_dev entries of order: the visible pairs), and the tiles of every
+// entry in that order: the scan below reads them where it writes its offsets,
+// so that the gather is done once.
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_reduce(const uint32_t* __restrict__ order, const uint32_t* __restrict__ touched,
-              const uint32_t* count_dev, uint32_t* __restrict__ block_sums) {
+              const uint32_t* count_dev, uint32_t* __restrict__ block_sums,
+              uint32_t* __restrict__ tiles_of) {
     grid_dep_begin();
     __shared__ uint32_t wt[33];
     const uint32_t count = *count_dev;
     const uint32_t start = blockIdx.x * (uint32_t)kScanTile;
-    uint32_t s = 0;
+    if (start >= count) return;  // (its sum is never read)
+    uint32_t t[kScanItems], s = 0;
+#pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        const uint32_t i = start + threadIdx.x * kScanItems + k;
-        if (i < count) s += touched[order[i]];
+        const uint32_t i = start + k * kScanThreads + threadIdx.x;
+        t[k] = i < count ? touched[order[i]] : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        const uint32_t i = start + k * kScanThreads + threadIdx.x;
+        if (i < count) tiles_of[i] = t[k];
+        s += t[k];
     }
     uint32_t tot;
     block_exclusive_scan(s, wt, tot);
@@ -263,13 +391,15 @@ __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long x
 // block sums runs; CTA 0 also forms the total and the instance counters
 // (vn = the number of depth-order entries, for later readers).
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_offsets(const uint32_t* __restrict__ order, const uint32_t* __restrict__ touched,
-               const uint32_t* __restrict__ block_sums, int nb, uint32_t cap,
+k_scan_offsets(const uint32_t* __restrict__ block_sums, uint32_t cap,
                const uint32_t* count_dev, DevCounters* ctr, uint32_t* __restrict__ off) {
     grid_dep_begin();
     __shared__ uint32_t wt[33];
     __shared__ unsigned long long red[kScanThreads / 32];
     const uint32_t count = *count_dev;
+    const uint32_t start = blockIdx.x * (uint32_t)kScanTile;
+    if (blockIdx.x > 0 && start >= count) return;
+    const int nb = (int)((count + kScanTile - 1) / kScanTile);
     unsigned long long pre = 0;
     for (int i = threadIdx.x; i < (int)blockIdx.x; i += blockDim.x) pre += block_sums[i];
     pre = block_sum_u64(pre, red);
@@ -284,23 +414,45 @@ k_scan_offsets(const uint32_t* __restrict__ order, const uint32_t* __restrict__ 
             if (tot > cap) atomicOr(&ctr->status, (uint32_t)GS_DEV_CAPACITY);
         }
     }
-    const uint32_t start = blockIdx.x * (uint32_t)kScanTile;
+    // off holds the entries' tiles (k_scan_reduce) and becomes their offsets
+    const uint32_t i0 = start + threadIdx.x * kScanItems;
     uint32_t t[kScanItems], s = 0;
-    for (int k = 0; k < kScanItems; ++k) {
-        const uint32_t i = start + threadIdx.x * kScanItems + k;
-        t[k] = i < count ? touched[order[i]] : 0u;
-        s += t[k];
+    static_assert(kScanItems % 4 == 0, "whole 16-byte groups of offsets");
+    const bool whole = i0 + kScanItems <= count;
+    if (whole) {
+#pragma unroll
+        for (int k = 0; k < kScanItems; k += 4) {
+            const uint4 x = *reinterpret_cast<const uint4*>(off + i0 + k);
+            t[k] = x.x;
+            t[k + 1] = x.y;
+            t[k + 2] = x.z;
+            t[k + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) t[k] = i0 + k < count ? off[i0 + k] : 0u;
     }
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) s += t[k];
     uint32_t tot;
     unsigned long long o = pre + block_exclusive_scan(s, wt, tot);
     auto word = [](unsigned long long x) { return (uint32_t)min(x, 0xFFFFFFFFull); };
+#pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        const uint32_t i = start + threadIdx.x * kScanItems + k;
-        if (i < count) {
-            off[i] = word(o);
-            if (i + 1 == count) off[count] = word(o + t[k]);  // the total
-        }
-        o += t[k];
+        const uint32_t tiles = t[k];
+        t[k] = word(o);
+        o += tiles;
+        if (i0 + k + 1 == count) off[count] = word(o);  // the total
+    }
+    if (whole) {
+#pragma unroll
+        for (int k = 0; k < kScanItems; k += 4)
+            *reinterpret_cast<uint4*>(off + i0 + k) =
+                make_uint4(t[k], t[k + 1], t[k + 2], t[k + 3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k)
+            if (i0 + k < count) off[i0 + k] = t[k];
     }
 }
 
@@ -550,51 +702,61 @@ k_tile_order(const uint32_t* __restrict__ ranges, int T, const uint32_t* __restr
 // is counted on the device launch this many at most, so that no CTA is
 // launched only to find nothing to do.
 template <auto Kernel>
-int resident_grid(int threads) {
-    static std::atomic<int> per_sm{0};
-    int b = per_sm.load(std::memory_order_relaxed);
-    if (b <= 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, Kernel, threads, 0) !=
+int resident_grid(int threads, size_t smem = 0) {
+    // (a kernel's launches differ in shared memory by its digits: the last
+    // asked for is kept)
+    static std::atomic<unsigned long long> known{~0ull};
+    const unsigned long long k0 = known.load(std::memory_order_relaxed);
+    int b = (int)(k0 >> 32);
+    if (k0 == ~0ull || (k0 & 0xFFFFFFFFull) != smem) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, Kernel, threads, smem) !=
                 cudaSuccess ||
             b < 1)
             b = 1;
-        per_sm.store(b, std::memory_order_relaxed);
+        known.store((unsigned long long)b << 32 | smem, std::memory_order_relaxed);
     }
     return b * sm_count();
 }
 
+// One stable pass over up to `cap` keys (the real count comes from count_dev
+// when given).  digits: the most the pass can have.  With kept_out the pass
+// drops the culled keys and stores how many it kept there.
 template <int ITEMS>
 gs_status radix_pass_t(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
-                       const uint32_t* count_dev, uint32_t count_host, uint32_t cap, int shift,
-                       int bits, uint32_t* hist, uint32_t* totals, uint32_t* kept_out,
+                       const uint32_t* count_dev, uint32_t count_host, uint32_t cap, Digit dg,
+                       int digits, uint32_t* hist, uint32_t* totals, uint32_t* kept_out,
                        cudaStream_t st) {
     const int nb = (int)((cap + kSortThreads * ITEMS - 1) / (kSortThreads * ITEMS));
     const int drop = kept_out != nullptr;
-    const uint32_t mask = (1u << bits) - 1u;
-    const int hg = min(nb, resident_grid<k_radix_hist<ITEMS>>(kSortThreads));
-    const int sg = min(nb, resident_grid<k_radix_scatter<ITEMS>>(kSortThreads));
-    launch_pdl(k_radix_hist<ITEMS>, hg, kSortThreads, 0, st, kin, count_dev, count_host, cap,
-               shift, mask, nb, drop, hist);
-    launch_pdl(k_radix_scan<ITEMS>, kRadix, kSortThreads, 0, st, hist, count_dev, count_host,
-               cap, nb, totals);
-    launch_pdl(k_radix_scatter<ITEMS>, sg, kSortThreads, 0, st, kin, vin, kout, vout, count_dev,
-               count_host, cap, shift, mask, nb, hist, totals, drop, kept_out);
+    const size_t hs = (size_t)digits * 4, ss = scatter_smem(digits, ITEMS);
+    if (cudaFuncSetAttribute(k_radix_scatter<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)scatter_smem(kDigits, ITEMS)) != cudaSuccess)
+        return GS_ERR_CUDA;
+    const int hg = min(nb, resident_grid<k_radix_hist<ITEMS>>(kSortThreads, hs));
+    const int sg = min(nb, resident_grid<k_radix_scatter<ITEMS>>(kSortThreads, ss));
+    const int cg = min(digits, resident_grid<k_radix_scan<ITEMS>>(kScanThreads));
+    launch_pdl(k_radix_hist<ITEMS>, hg, kSortThreads, hs, st, kin, count_dev, count_host, cap, dg,
+               nb, drop, hist);
+    launch_pdl(k_radix_scan<ITEMS>, cg, kScanThreads, 0, st, hist, count_dev, count_host, cap, dg,
+               nb, totals);
+    launch_pdl(k_radix_scatter<ITEMS>, sg, kSortThreads, ss, st, kin, vin, kout, vout, count_dev,
+               count_host, cap, dg, nb, hist, totals, drop, kept_out);
     return launch_status();
 }
 
-// One stable pass on `bits` (<= 8) bits at `shift` over up to `cap` keys (the real count
-// comes from count_dev when given), in blocks of 1024 keys: measured faster
-// than blocks of 2048 or 4096 for both the 1M depth keys and the 5M instances
-// (with the digit-reordered, coalesced writes too).  With kept_out the pass
-// drops the culled keys and stores how many it kept there.
-template <int ITEMS = kSortItems>
+// Blocks of 1024 keys where they are needed to have enough of them (200k pairs,
+// 150k instances: whole binning 52 us, 58 with 2048), of 2048 from kSortLarge
+// keys on, half the histogram (13.8M instances 632 us, 732 with 1024, 656 with
+// 3072, all with 8-bit digits).
 gs_status radix_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
-                     const uint32_t* count_dev, uint32_t count_host, uint32_t cap, int shift,
-                     int bits, uint32_t* hist, uint32_t* totals, cudaStream_t st,
+                     const uint32_t* count_dev, uint32_t count_host, uint32_t cap, Digit dg,
+                     int digits, uint32_t* hist, uint32_t* totals, cudaStream_t st,
                      uint32_t* kept_out = nullptr) {
-    static_assert(ITEMS >= kSortItems, "the histogram buffer holds kSortTile-key blocks");
-    return radix_pass_t<ITEMS>(kin, vin, kout, vout, count_dev, count_host, cap, shift, bits,
-                               hist, totals, kept_out, st);
+    return cap < kSortLarge
+               ? radix_pass_t<kSortItems>(kin, vin, kout, vout, count_dev, count_host, cap, dg,
+                                          digits, hist, totals, kept_out, st)
+               : radix_pass_t<kSortItemsLarge>(kin, vin, kout, vout, count_dev, count_host, cap,
+                                               dg, digits, hist, totals, kept_out, st);
 }
 
 }  // namespace
@@ -603,36 +765,38 @@ gs_status radix_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, u
 static gs_status depth_sort(const Plan* p, uint32_t VN, uint32_t icap, void* ws, uint32_t* hist,
                             uint32_t* totals, cudaStream_t st) {
     DevCounters* ctr = buf<DevCounters>(p, ws, GS_BUF_COUNTERS);
-    // 1. depth digits over the (view, Gaussian) pairs: 4 passes, the
-    //    projection's keys (values = positions) -> B -> C -> B -> C; the first
-    //    keeps only the visible pairs, whose count (n_sorted) the later passes
-    //    read on the device.  The projection's keys are left intact, so a
+    // 1. depth digits over the (view, Gaussian) pairs: 3 passes, the
+    //    projection's keys (values = positions) -> C -> B -> the depth order; the
+    //    first keeps only the visible pairs, whose count (n_sorted) the later
+    //    passes read on the device.  The projection's keys are left intact, so a
     //    second binning of the same projection sorts the same pairs.
-    const uint32_t* kp = buf<uint32_t>(p, ws, B_DKEY_A);
     uint32_t* kb = buf<uint32_t>(p, ws, B_DKEY_B);
     uint32_t* vb = buf<uint32_t>(p, ws, B_DVAL_B);
     uint32_t* kc = buf<uint32_t>(p, ws, B_DKEY_C);
     uint32_t* va = buf<uint32_t>(p, ws, GS_BUF_DEPTH_ORDER);
     uint32_t* n_sorted = &ctr->n_sorted;
-    gs_status s = radix_pass(kp, nullptr, kb, vb, nullptr, VN, VN, 0, kRadixBits, hist, totals,
-                              st, n_sorted);
+    Digit dg = {ctr, 0u, 0, 0};
+    const float near_z = p->cfg.near_z;
+    __builtin_memcpy(&dg.sub, &near_z, sizeof(near_z));
+    gs_status s = radix_pass(buf<uint32_t>(p, ws, B_DKEY_A), nullptr, kc, va, nullptr, VN, VN, dg,
+                             kDigits, hist, totals, st, n_sorted);
     if (s != GS_OK) return s;
-    for (int pass = 1; pass < 4; ++pass) {
-        const bool odd = (pass & 1) != 0;
-        s = radix_pass(odd ? kb : kc, odd ? vb : va, odd ? kc : kb, odd ? va : vb,
-                                 n_sorted, VN, VN, pass * kRadixBits, kRadixBits, hist, totals,
-                                 st);
-        if (s != GS_OK) return s;
-    }
+    static_assert(kDepthPasses == 3, "two more passes, the last without keys");
+    dg.shift = 1;
+    s = radix_pass(kc, va, kb, vb, n_sorted, VN, VN, dg, kDigits, hist, totals, st);
+    if (s != GS_OK) return s;
+    dg.shift = 2;
+    s = radix_pass(kb, vb, nullptr, va, n_sorted, VN, VN, dg, kDigits, hist, totals, st);
+    if (s != GS_OK) return s;
 
     // 2. scan of tiles touched in depth order (grids over all pairs; blocks past
     //    the visible count do nothing)
     const int snb = (int)((VN + kScanTile - 1) / kScanTile);
     uint32_t* bsums = buf<uint32_t>(p, ws, B_SCAN_BLOCKS);
     const uint32_t* touched = buf<uint32_t>(p, ws, GS_BUF_TOUCHED);
-    launch_pdl(k_scan_reduce, snb, kScanThreads, 0, st, va, touched, n_sorted, bsums);
-    launch_pdl(k_scan_offsets, snb, kScanThreads, 0, st, va, touched, bsums, snb, icap, n_sorted,
-               ctr, buf<uint32_t>(p, ws, B_OFFSETS));
+    uint32_t* offs = buf<uint32_t>(p, ws, B_OFFSETS);
+    launch_pdl(k_scan_reduce, snb, kScanThreads, 0, st, va, touched, n_sorted, bsums, offs);
+    launch_pdl(k_scan_offsets, snb, kScanThreads, 0, st, bsums, icap, n_sorted, ctr, offs);
     return launch_status();
 }
 
@@ -644,9 +808,7 @@ gs_status launch_bin_sort(const Plan* p, int32_t n, void* ws, cudaStream_t st) {
     const uint32_t VN = (uint32_t)p->vt.n_views * (uint32_t)n;
     const uint32_t icap = (uint32_t)p->inst_capacity;
     uint32_t* hist = buf<uint32_t>(p, ws, B_HIST);
-    uint32_t* totals = hist + (size_t)kRadix * (p->depth_sort_blocks > p->inst_sort_blocks
-                                                    ? p->depth_sort_blocks
-                                                    : p->inst_sort_blocks);
+    uint32_t* totals = hist + p->hist_words;
     DevCounters* ctr = buf<DevCounters>(p, ws, GS_BUF_COUNTERS);
     // the per-tile ranges are cleared first, so that every kernel of the
     // binning follows another kernel (programmatic launches, see launch_pdl);
@@ -683,8 +845,9 @@ gs_status launch_bin_sort(const Plan* p, int32_t n, void* ws, cudaStream_t st) {
     const int tbits = (p->tile_bits + p->tile_passes - 1) / p->tile_passes;
     for (int pass = 0; pass < p->tile_passes; ++pass) {
         const bool even = (pass & 1) == 0;
+        const Digit dg = {nullptr, 0u, pass * tbits, tbits};
         s = radix_pass(even ? ika : ikb, even ? iva : ivb, even ? ikb : ika, even ? ivb : iva, cnt,
-                       0u, icap, pass * tbits, tbits, hist, totals, st);
+                       0u, icap, dg, 1 << tbits, hist, totals, st);
         if (s != GS_OK) return s;
     }
     const uint32_t* sorted_keys = (p->tile_passes & 1) ? ikb : ika;
