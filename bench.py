@@ -77,7 +77,7 @@ def iteration_roofline(n, sh_degree, n_views, n_values, n_pixels, instances, pai
     vn = n_views * n
     stages = dict(
         project=((n_views + 3) // 4 * n * pb + vn * 72) / bw,
-        bin_sort=(vn * (4 * 16 + 12) + instances * (8 + 16 * passes + 4) + tiles * 8) / bw,
+        bin_sort=(vn * (4 * 12 + 12) + instances * (8 + 16 * passes + 4) + tiles * 8) / bw,
         render_fwd=max(pairs * PAIR_FLOPS_FWD / fl, (instances * 48 + n_pixels * 20) / bw),
         loss_l1_ssim=n_values * 44 / bw,
         render_bwd=max(pairs * PAIR_FLOPS_BWD / fl, (instances * 48 + n_pixels * 16) / bw),

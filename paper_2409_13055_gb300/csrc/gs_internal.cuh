@@ -71,7 +71,6 @@ enum PrivBuf {
     B_IVAL_B,
     B_LOSS_MAPS,
     B_LOSS_BLOCKS,
-    B_GCOL,     // [V*n] x 3: colour gradient as it reaches the SH coefficients
     B_OFFSETS,  // [V*n + 1] instance offsets of the entries in depth order
     B_TILE_ORDER,  // [total_tiles] render order of the tiles, longest lists first;
                    // then 2 x kOrderBuckets words of scratch for building it

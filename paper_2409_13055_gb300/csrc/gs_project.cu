@@ -536,14 +536,14 @@ __device__ __forceinline__ bool group_touched(int g, int n, int n_views,
 // quaternion and opacity logit.  The colour gradient that reaches the SH
 // coefficients (zero on clamped channels, a grayscale view's gradient spread
 // over the three channels) goes, by MODE:
-//   kShViaGcol  to gcol_out per (view, Gaussian), for k_sh_bwd;
 //   kShStaged   into this Gaussian's SH gradient at once, sh_acc[k * sh_stride
-//               + c] += Y_k(dir) gcol[c] view by view in view order (the sum
-//               k_sh_bwd forms), sh_acc in shared memory;
+//               + c] += Y_k(dir) gcol[c] view by view in view order, sh_acc in
+//               shared memory;
 //   kShDirect   (one view only) straight to the SH gradient array, sh_acc =
 //               its row of this Gaussian, sh_stride = 3 n: Y_k(dir) gcol[c],
-//               rounded as k_sh_bwd rounds it, written or (accumulate) added.
-constexpr int kShViaGcol = 0, kShStaged = 1, kShDirect = 2;
+//               rounded as the staged sum's only term, written or (accumulate)
+//               added.
+constexpr int kShStaged = 1, kShDirect = 2;
 
 template <int DEG, int MODE>
 __device__ __forceinline__ void adjoint_one(
@@ -551,7 +551,7 @@ __device__ __forceinline__ void adjoint_one(
     const float* __restrict__ quats, const float* __restrict__ opacity_logits,
     const float* __restrict__ sh, int n, const Cam* cam_all, const ViewTable& vt, float near_z,
     const uint32_t* __restrict__ touched, const float* __restrict__ grad2d,
-    float* __restrict__ gcol_out, float* sh_acc, size_t sh_stride, int accumulate,
+    float* sh_acc, size_t sh_stride, int accumulate,
     float gm_out[3], float gls[3], float4& gq4, float& glog) {
     const float mean[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
     const float ls[3] = {log_scales[3 * g], log_scales[3 * g + 1], log_scales[3 * g + 2]};
@@ -585,13 +585,7 @@ __device__ __forceinline__ void adjoint_one(
         Proj p;
         project_one(mean, shp, cam, near_z, vt.log2_tw, vt.log2_th, geo.tiles_x, geo.tiles_y,
                     opacity, vt.tight_rect, p);
-        if (!p.visible) {
-            if (MODE == kShViaGcol) {
-                float* gc_out = gcol_out + vg * 3;
-                gc_out[0] = gc_out[1] = gc_out[2] = 0.0f;
-            }
-            continue;
-        }
+        if (!p.visible) continue;
 
         gop += gO;
         // colour -> SH coefficients and the viewing direction
@@ -619,7 +613,7 @@ __device__ __forceinline__ void adjoint_one(
                 a[1] = fmaf(Y[k], gcol[1], a[1]);
                 a[2] = fmaf(Y[k], gcol[2], a[2]);
             }
-        } else if (MODE == kShDirect) {
+        } else {
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 float* a = sh_acc + k * sh_stride;
@@ -630,11 +624,6 @@ __device__ __forceinline__ void adjoint_one(
                 }
             }
             sh_written = true;
-        } else {
-            float* gc_out = gcol_out + vg * 3;
-            gc_out[0] = gcol[0];
-            gc_out[1] = gcol[1];
-            gc_out[2] = gcol[2];
         }
         float w[16];
 #pragma unroll
@@ -751,22 +740,46 @@ __device__ __forceinline__ void adjoint_one(
 }
 
 
-// DIRECT (single-view plans): the SH gradient is written here and k_sh_bwd
-// is not launched.  With group_vis, a warp's 32 Gaussians form a group: a
+// Where the gradients of the four geometry groups go, written or (accumulate) added.
+__device__ __forceinline__ void put_geometry(int g, const float* gm, const float* gls,
+                                             const float4& gq4, float glog,
+                                             float* __restrict__ g_means, float* __restrict__ g_ls,
+                                             float* __restrict__ g_quats,
+                                             float* __restrict__ g_logit, int accumulate) {
+    if (accumulate) {
+        for (int e = 0; e < 3; ++e) {
+            g_means[3 * g + e] += gm[e];
+            g_ls[3 * g + e] += gls[e];
+        }
+        float4 o = reinterpret_cast<float4*>(g_quats)[g];
+        o.x += gq4.x; o.y += gq4.y; o.z += gq4.z; o.w += gq4.w;
+        reinterpret_cast<float4*>(g_quats)[g] = o;
+        g_logit[g] += glog;
+    } else {
+        for (int e = 0; e < 3; ++e) {
+            g_means[3 * g + e] = gm[e];
+            g_ls[3 * g + e] = gls[e];
+        }
+        reinterpret_cast<float4*>(g_quats)[g] = gq4;
+        g_logit[g] = glog;
+    }
+}
+
+// Single-view plans.  With group_vis, a warp's 32 Gaussians form a group: a
 // group none of whose Gaussians touches a tile in any view (all-zero
 // gradient) writes nothing, and group_vis[group] records which groups wrote.
-template <int DEG, bool DIRECT>
+template <int DEG>
 __global__ void __launch_bounds__(kProjThreads, 2)
 k_project_bwd(const float* __restrict__ means, const float* __restrict__ log_scales,
               const float* __restrict__ quats, const float* __restrict__ opacity_logits,
               const float* __restrict__ sh, int n, const gs_view* __restrict__ views,
               ViewTable vt, float near_z, const uint32_t* __restrict__ touched,
-              const float* __restrict__ grad2d, float* __restrict__ gcol_out,
+              const float* __restrict__ grad2d,
               float* __restrict__ g_means, float* __restrict__ g_ls, float* __restrict__ g_quats,
               float* __restrict__ g_logit, float* __restrict__ g_sh, int accumulate,
               uint8_t* __restrict__ group_vis) {
-    extern __shared__ Cam cam_all[];
-    for (int v = threadIdx.x; v < vt.n_views; v += blockDim.x) load_cam(views[v], cam_all[v]);
+    __shared__ Cam cam;
+    if (threadIdx.x == 0) load_cam(views[0], cam);
     __syncthreads();
     // a grid of resident CTAs striding over the Gaussians (whole warps: the
     // group vote stays warp-wide); a thread's next Gaussian's touched words
@@ -775,87 +788,108 @@ k_project_bwd(const float* __restrict__ means, const float* __restrict__ log_sca
     for (int g0 = blockIdx.x * blockDim.x; g0 < n; g0 += stride) {
         const int g = g0 + threadIdx.x;
         if (g + stride < n) {
-            for (int v = 0; v < vt.n_views; ++v)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(touched + (size_t)v * n + g + stride));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(touched + g + stride));
             prefetch_params(means, log_scales, quats, opacity_logits, g + stride);
         }
-        if (group_vis && !group_touched(g, n, vt.n_views, touched, group_vis)) continue;
+        if (group_vis && !group_touched(g, n, 1, touched, group_vis)) continue;
         if (g >= n) continue;
         float gm[3], gls[3], glog;
         float4 gq4;
-        adjoint_one<DEG, DIRECT ? kShDirect : kShViaGcol>(
-            g, means, log_scales, quats, opacity_logits, sh, n, cam_all, vt, near_z, touched, grad2d,
-            gcol_out, DIRECT ? g_sh + (size_t)g * 3 : nullptr, (size_t)3 * n, accumulate, gm, gls,
-            gq4, glog);
-        if (accumulate) {
-            for (int e = 0; e < 3; ++e) {
-                g_means[3 * g + e] += gm[e];
-                g_ls[3 * g + e] += gls[e];
-            }
-            float4 o = reinterpret_cast<float4*>(g_quats)[g];
-            o.x += gq4.x; o.y += gq4.y; o.z += gq4.z; o.w += gq4.w;
-            reinterpret_cast<float4*>(g_quats)[g] = o;
-            g_logit[g] += glog;
-        } else {
-            for (int e = 0; e < 3; ++e) {
-                g_means[3 * g + e] = gm[e];
-                g_ls[3 * g + e] = gls[e];
-            }
-            reinterpret_cast<float4*>(g_quats)[g] = gq4;
-            g_logit[g] = glog;
-        }
+        adjoint_one<DEG, kShDirect>(
+            g, means, log_scales, quats, opacity_logits, sh, n, &cam, vt, near_z, touched, grad2d,
+            g_sh + (size_t)g * 3, (size_t)3 * n, accumulate, gm, gls, gq4, glog);
+        put_geometry(g, gm, gls, gq4, glog, g_means, g_ls, g_quats, g_logit, accumulate);
     }
 }
 
-// Gradient of the SH coefficients: sum over views of Y_k(dir_v) gcol_v, with
-// gcol the colour gradient k_project_bwd left (zero on clamped channels, a
-// grayscale view's gradient spread over the three channels).
+// Plans of several views: the SH gradient is summed over the views in shared
+// memory, [K][3 T] in the order of the gradient array, and a warp then writes its
+// 32 Gaussians' run of every coefficient plane as three 128-byte lines (adding to
+// what is there, kPlanes planes' loads in flight).  When it adds, a Gaussian that
+// no view of the pass touches is left out altogether: its gradient is zero.  (Not
+// one whose parameters overflow or are not finite: its zeros become NaN on the
+// way, and are added.)  The groups as above.  Bound by latency at the 16 warps
+// per SM that 128 registers leave (16 views) and by the gradients' bytes (two
+// views of 2M).  The colour gradients used to go through memory to a second
+// kernel for the SH sums, a thread per Gaussian reading and writing 12 of every
+// 384 bytes a plane: 16 views of 500k 285 -> 212 us, two views of 2M 287 -> 262.
+// CTAs of 128 threads, one per 128 Gaussians: resident ones that stride end
+// unevenly (223 us).
+constexpr int kViewsThreads = 128;
+
 template <int DEG>
-__global__ void __launch_bounds__(kProjThreads)
-k_sh_bwd(const float* means, int n, const gs_view* __restrict__ views, ViewTable vt,
-         const uint32_t* __restrict__ touched, const float* __restrict__ gcol_in,
-         float* __restrict__ g_sh, int accumulate, int groups) {
-    extern __shared__ Cam cam_all[];
-    for (int v = threadIdx.x; v < vt.n_views; v += blockDim.x) load_cam(views[v], cam_all[v]);
+__global__ void __launch_bounds__(kViewsThreads, 4)
+k_project_bwd_views(const float* __restrict__ means, const float* __restrict__ log_scales,
+                    const float* __restrict__ quats, const float* __restrict__ opacity_logits,
+                    const float* __restrict__ sh, int n, const gs_view* __restrict__ views,
+                    ViewTable vt, float near_z, const uint32_t* __restrict__ touched,
+                    const float* __restrict__ grad2d,
+                    float* __restrict__ g_means, float* __restrict__ g_ls,
+                    float* __restrict__ g_quats, float* __restrict__ g_logit,
+                    float* __restrict__ g_sh, int accumulate, uint8_t* __restrict__ group_vis,
+                    const DevCounters* __restrict__ ctr) {
+    constexpr int K = (DEG + 1) * (DEG + 1), T = kViewsThreads;
+    constexpr int kPlanes = K % 4 == 0 ? 4 : K % 3 == 0 ? 3 : 1;
+    extern __shared__ float stage[];
+    Cam* const cam_all = reinterpret_cast<Cam*>(stage + 3 * K * T);
+    for (int v = threadIdx.x; v < vt.n_views; v += T) load_cam(views[v], cam_all[v]);
     __syncthreads();
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (groups && !group_touched(g, n, vt.n_views, touched, nullptr)) return;
-    if (g >= n) return;
-    constexpr int K = (DEG + 1) * (DEG + 1);
-    const float mean[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
-    float acc[K][3];
-#pragma unroll
-    for (int k = 0; k < K; ++k) acc[k][0] = acc[k][1] = acc[k][2] = 0.0f;
-    for (int v = 0; v < vt.n_views; ++v) {
-        const size_t vg = (size_t)v * n + g;
-        if (touched[vg] == 0u) continue;
-        const float* gc = gcol_in + vg * 3;
-        const float c0 = gc[0], c1 = gc[1], c2 = gc[2];
-        const Cam& cam = cam_all[v];
-        const float d0 = mean[0] - cam.cc[0], d1 = mean[1] - cam.cc[1], d2 = mean[2] - cam.cc[2];
-        const float dist = sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
-        const float id = dist > 0.0f ? 1.0f / dist : 0.0f;
-        float Y[16];
-        sh_eval(DEG, d0 * id, d1 * id, d2 * id, Y);
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            acc[k][0] = fmaf(Y[k], c0, acc[k][0]);
-            acc[k][1] = fmaf(Y[k], c1, acc[k][1]);
-            acc[k][2] = fmaf(Y[k], c2, acc[k][2]);
+    const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
+    float* const mine = stage + 3 * w0;  // the warp's run of a plane
+    const bool clean = (ctr->status & (uint32_t)GS_DEV_NONFINITE) == 0u;
+    // (one turn with the grid that is launched; without the loop ptxas spills six
+    // times as much at degree 3)
+    for (int g0 = blockIdx.x * T; g0 + w0 < n; g0 += gridDim.x * T) {
+        const int g = g0 + threadIdx.x;
+        bool reached = false;
+        if (g < n)
+            for (int v = 0; v < vt.n_views; ++v) reached |= touched[(size_t)v * n + g] != 0u;
+        const bool any = __any_sync(0xffffffffu, reached);
+        if (group_vis) {
+            if (lane == 0) group_vis[g >> 5] = any ? 1 : 0;
+            if (!any) continue;
         }
-    }
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        float* o = g_sh + ((size_t)k * n + g) * 3;
-        if (accumulate) {
-            o[0] += acc[k][0];
-            o[1] += acc[k][1];
-            o[2] += acc[k][2];
-        } else {
-            o[0] = acc[k][0];
-            o[1] = acc[k][1];
-            o[2] = acc[k][2];
+        bool live = g < n;
+        if (accumulate && clean && live && !reached) {
+            const float most =
+                fmaxf(log_scales[3 * g], fmaxf(log_scales[3 * g + 1], log_scales[3 * g + 2]));
+            live = !(most < 40.0f);  // (its square is finite)
         }
+        const unsigned who = __ballot_sync(0xffffffffu, live);
+        if (who == 0u) continue;
+#pragma unroll
+        for (int k = 0; k < 3 * K; ++k) mine[(k / 3) * 3 * T + (k % 3) * 32 + lane] = 0.0f;
+        __syncwarp();
+        if (live) {
+            float gm[3], gls[3], glog;
+            float4 gq4;
+            adjoint_one<DEG, kShStaged>(g, means, log_scales, quats, opacity_logits, sh, n,
+                                        cam_all, vt, near_z, touched, grad2d, mine + 3 * lane,
+                                        3 * T, 0, gm, gls, gq4, glog);
+            put_geometry(g, gm, gls, gq4, glog, g_means, g_ls, g_quats, g_logit, accumulate);
+        }
+        __syncwarp();
+        float* const out = g_sh + (size_t)3 * (g0 + w0) + lane;
+        bool put[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) put[j] = (who >> ((lane + 32 * j) / 3)) & 1u;
+        for (int k = 0; k < K; k += kPlanes) {
+            float o[kPlanes][3];
+#pragma unroll
+            for (int q = 0; q < kPlanes; ++q)
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    o[q][j] = accumulate && put[j] ? out[(size_t)(k + q) * 3 * n + 32 * j] : 0.0f;
+#pragma unroll
+            for (int q = 0; q < kPlanes; ++q)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const float a = mine[(k + q) * 3 * T + 32 * j + lane];
+                    if (put[j])
+                        out[(size_t)(k + q) * 3 * n + 32 * j] = accumulate ? o[q][j] + a : a;
+                }
+        }
+        __syncwarp();
     }
 }
 
@@ -1000,7 +1034,7 @@ k_adjoint_adam(const float* __restrict__ means, const float* __restrict__ log_sc
         float gm[3], gls[3], glog;
         float4 gq4;
         adjoint_one<DEG, kShStaged>(g0 + t, means, log_scales, quats, opacity_logits, sh, n,
-                                    cam_all, vt, near_z, touched, grad2d, nullptr, sh_acc, 3 * C,
+                                    cam_all, vt, near_z, touched, grad2d, sh_acc, 3 * C,
                                     0, gm, gls, gq4, glog);
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
@@ -1080,45 +1114,38 @@ gs_status launch_project(const Plan* p, const gs_map* map, const gs_view* views_
     return launch_status();
 }
 
-static gs_status launch_project_adjoint(const Plan* p, const gs_map* map,
-                                        const gs_view* views_dev, void* ws,
-                                        const gs_map_grad* grads, int accumulate,
-                                        uint8_t* group_vis, cudaStream_t st) {
-    const int n = map->n;
-    const size_t smem = sizeof(Cam) * p->vt.n_views;
-    const bool direct = p->vt.n_views == 1;
-    auto* kern = direct ? (map->sh_degree == 0   ? k_project_bwd<0, true>
-                           : map->sh_degree == 1 ? k_project_bwd<1, true>
-                           : map->sh_degree == 2 ? k_project_bwd<2, true>
-                                                 : k_project_bwd<3, true>)
-                        : (map->sh_degree == 0   ? k_project_bwd<0, false>
-                           : map->sh_degree == 1 ? k_project_bwd<1, false>
-                           : map->sh_degree == 2 ? k_project_bwd<2, false>
-                                                 : k_project_bwd<3, false>);
-    const int blocks =
-        resident_grid(kern, kProjThreads, smem, (n + kProjThreads - 1) / kProjThreads);
-    kern<<<blocks, kProjThreads, smem, st>>>(
-        map->means, map->log_scales, map->quats, map->opacity_logits, map->sh, n, views_dev,
-        p->vt, p->cfg.near_z, buf<uint32_t>(p, ws, GS_BUF_TOUCHED),
-        buf<float>(p, ws, GS_BUF_GRAD2D), buf<float>(p, ws, B_GCOL), grads->means,
-        grads->log_scales, grads->quats, grads->opacity_logits, grads->sh, accumulate, group_vis);
-    return launch_status();
-}
-
 gs_status launch_project_bwd(const Plan* p, const gs_map* map, const gs_view* views_dev,
                              void* ws, const gs_map_grad* grads, int accumulate,
                              cudaStream_t st, uint8_t* group_vis) {
     if (reinterpret_cast<uintptr_t>(grads->quats) % 16) return GS_ERR_INVALID;
-    gs_status s = launch_project_adjoint(p, map, views_dev, ws, grads, accumulate, group_vis, st);
-    if (s != GS_OK || p->vt.n_views == 1) return s;  // one view: SH gradient already written
     const int n = map->n;
-    auto* kern_sh = map->sh_degree == 0   ? k_sh_bwd<0>
-                    : map->sh_degree == 1 ? k_sh_bwd<1>
-                    : map->sh_degree == 2 ? k_sh_bwd<2>
-                                          : k_sh_bwd<3>;
-    kern_sh<<<(n + kProjThreads - 1) / kProjThreads, kProjThreads, sizeof(Cam) * p->vt.n_views,
-              st>>>(map->means, n, views_dev, p->vt, buf<uint32_t>(p, ws, GS_BUF_TOUCHED),
-                    buf<float>(p, ws, B_GCOL), grads->sh, accumulate, group_vis ? 1 : 0);
+    const uint32_t* touched = buf<uint32_t>(p, ws, GS_BUF_TOUCHED);
+    const float* grad2d = buf<float>(p, ws, GS_BUF_GRAD2D);
+    if (p->vt.n_views == 1) {
+        auto* kern = map->sh_degree == 0   ? k_project_bwd<0>
+                     : map->sh_degree == 1 ? k_project_bwd<1>
+                     : map->sh_degree == 2 ? k_project_bwd<2>
+                                           : k_project_bwd<3>;
+        const int blocks =
+            resident_grid(kern, kProjThreads, 0, (n + kProjThreads - 1) / kProjThreads);
+        kern<<<blocks, kProjThreads, 0, st>>>(
+            map->means, map->log_scales, map->quats, map->opacity_logits, map->sh, n, views_dev,
+            p->vt, p->cfg.near_z, touched, grad2d, grads->means, grads->log_scales, grads->quats,
+            grads->opacity_logits, grads->sh, accumulate, group_vis);
+        return launch_status();
+    }
+    auto* kern = map->sh_degree == 0   ? k_project_bwd_views<0>
+                 : map->sh_degree == 1 ? k_project_bwd_views<1>
+                 : map->sh_degree == 2 ? k_project_bwd_views<2>
+                                       : k_project_bwd_views<3>;
+    const int K = (map->sh_degree + 1) * (map->sh_degree + 1);
+    const size_t smem = sizeof(float) * 3 * K * kViewsThreads + sizeof(Cam) * p->vt.n_views;
+    const int needed = (n + kViewsThreads - 1) / kViewsThreads;
+    kern<<<needed, kViewsThreads, smem, st>>>(
+        map->means, map->log_scales, map->quats, map->opacity_logits, map->sh, n, views_dev, p->vt,
+        p->cfg.near_z, touched, grad2d, grads->means, grads->log_scales, grads->quats,
+        grads->opacity_logits, grads->sh, accumulate, group_vis,
+        buf<DevCounters>(p, ws, GS_BUF_COUNTERS));
     return launch_status();
 }
 
