@@ -53,14 +53,13 @@ WORKLOAD = "room1M_1200x680"
 PAIR_FLOPS_FWD = 20.0
 PAIR_FLOPS_BWD = 60.0
 
-# DRAM bytes (read + write) of one k_render_bwd launch on the 1M 1200x680
-# workload stored in Z-order, from one single-pass ncu capture per launch
-# shape (tile, backward batch, backward pixels per thread) and tile-rect mode
-# of the kernel as committed; other shapes and modes report null.  The
-# capture's command and its other counters are kept with the launch-list
-# profile of this workload.
+# DRAM bytes (read + write) of one k_blocks_bwd launch on the 1M 1200x680
+# workload stored in Z-order, from an ncu capture of the kernel as committed,
+# by tile and tile-rect mode (batches and pixels per thread have no effect on
+# this kernel); others report null.  The capture's other counters are kept with
+# the profile of the block kernels.
 RENDER_BWD_TRAFFIC = {
-    ("room1M_1200x680", "8x8", 64, 2, "tight"): 54.52e6 + 0.02e6,
+    ("room1M_1200x680", "8x8", "tight"): 55.2e6,
 }
 
 
@@ -809,7 +808,6 @@ def run_gpu(args, ws, rank, local):
         traffic = None
         if dominant == "render_bwd" and args.map_order == "zorder" and not args.deterministic:
             traffic = RENDER_BWD_TRAFFIC.get((args.workload, f"{args.tile_w}x{args.tile_h}",
-                                              args.batch_bwd, args.ppt_bwd,
                                               "square" if args.square_rects else "tight"))
         roof = dict(bound="alu", kernel=dominant, achieved=achieved, peak=peak, unit="TFLOP/s",
                     frac=achieved / peak, traffic=traffic, algorithmic=flops,
