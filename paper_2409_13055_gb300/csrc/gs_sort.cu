@@ -729,9 +729,7 @@ gs_status radix_pass_t(const uint32_t* kin, const uint32_t* vin, uint32_t* kout,
     const int nb = (int)((cap + kSortThreads * ITEMS - 1) / (kSortThreads * ITEMS));
     const int drop = kept_out != nullptr;
     const size_t hs = (size_t)digits * 4, ss = scatter_smem(digits, ITEMS);
-    if (cudaFuncSetAttribute(k_radix_scatter<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)scatter_smem(kDigits, ITEMS)) != cudaSuccess)
-        return GS_ERR_CUDA;
+    static_assert(scatter_smem(kDigits, ITEMS) <= 48 * 1024, "no opt-in for shared memory");
     const int hg = min(nb, resident_grid<k_radix_hist<ITEMS>>(kSortThreads, hs));
     const int sg = min(nb, resident_grid<k_radix_scatter<ITEMS>>(kSortThreads, ss));
     const int cg = min(digits, resident_grid<k_radix_scan<ITEMS>>(kScanThreads));
