@@ -17,29 +17,27 @@
 //    evaluate alpha with the same rounded operations as gs_render.cu and take
 //    the same decisions.
 //  * The adjoint's sums over the block.  Per blended Gaussian the 64 pixels'
-//    dL/dpower and blend weights go to shared memory as one row of a window;
-//    eight rows make the A operand of mma.sync m16n8k8 (TF32 inputs, FP32
-//    sums), with each value split into two TF32 parts (rows 0-7 the high
-//    parts, rows 8-15 the low ones), against the monomials 1, x, y, x^2, xy,
-//    y^2 of the pixel's place in the block (exact in TF32) and against dL/dC
-//    (split the same way).  The moments about the Gaussian's mean follow from
-//    those about the block's centre.
+//    dL/dpower and blend weights go to shared memory as one row of a window; over
+//    eight rows a lane then sums the pixel pairs of one column of one row, and four
+//    lanes add up.  Products and sums are FP32, about the Gaussian's mean and in
+//    the order of the shuffles of gs_render.cu: an 8x8 tile's sums are the same
+//    bits as that kernel's.
 //
 // What bounds them: instruction issue and the ALU and heavy FMA pipes, two
 // cycles per instruction each (packed FP32 runs on the heavy pipe alone), and
 // for small launches the longest list, which one warp walks.  At 1M Gaussians,
 // 1200x680, 8x8 tiles (2.0M walked (block, Gaussian) pairs), against the kernels
-// of gs_render.cu at their best launch shape: forward 182 -> 131 us, 85 -> 51
-// warp instructions per pair; adjoint 319 -> 233 us, 138 -> 84.  Sixteen views of
-// a 500k map: 1003 -> 634 and 1593 -> 1318 us.  200k Gaussians, 640x480, 16x16
-// tiles: 68 -> 38 and 177 -> 77 us (there the block test and the four warps per
-// tile count as well).  What the adjoint gained by its parts at 1M: the window's
-// sums instead of shuffles 319 -> 265 us; a window row for every slot instead of
-// for the voted ones, so that the loop has no branch, 265 -> 241; that loop
-// unrolled over the window 241 -> 233.  Tried and not kept: the high parts rounded
-// instead of cut and a Newton step on 1 / (1 - alpha) (neither moved the
-// gradients' error against 64 bits), 32 slots per stage for a sixth CTA per SM (256
-// us).  In the forward, two pairs evaluated before a vote: 137 -> 131 us.
+// of gs_render.cu at their best launch shape: forward 182 -> 133 us, adjoint 319 ->
+// 253 us.  Sixteen views of a 500k map: 1003 -> 634 and 1593 -> 1332 us.  200k
+// Gaussians, 640x480, 16x16 tiles: 68 -> 38 and 177 -> 75 us (there the block test
+// and the four warps per tile count as well).
+//
+// The sums on mma.sync (TF32, each operand in two parts) take 233 us at 1M but
+// 77 at 200k, and two parts hold 22 bits of 24: every product came out low by 2e-7
+// on average, four times the rounding of the FP32 sums in the gradients of the SH
+// coefficients.  Tried and not kept: 32 slots per stage for a sixth CTA per SM (256
+// us against 241 then).  In the forward, two pairs evaluated before a vote: 137 ->
+// 131 us.
 #include "gs_render.cuh"
 
 namespace gs {
@@ -444,50 +442,28 @@ k_blocks_fwd(ViewTable vt, const uint32_t* __restrict__ ranges,
 // holds {dp, dp', w, w'} (both negated) at row_slot(r, e); the order within a row makes
 // the reads below free of bank conflicts.
 constexpr int kRows = 8;
-__device__ __forceinline__ int row_slot(int r, int e) {
-    const int c = e >> 3;
-    return r * 32 + (c << 3) + ((e & 7) ^ c ^ ((r & 1) << 2));
-}
-// ... and {|h_x|, |h_y|} of the density statistic, two lanes per float4.
-__device__ __forceinline__ int abs_slot(int r, int e2) {
-    const int c = e2 >> 2;
-    return r * 16 + (c << 2) + ((e2 & 3) ^ ((c >> 1) | ((r & 1) << 1)));
-}
+__device__ __forceinline__ int row_slot(int r, int e) { return r * 32 + (e ^ ((r & 1) << 2)); }
+// ... and {|h_x|, |h_y|} of the density statistic.
+__device__ __forceinline__ int abs_slot(int r, int e) { return r * 32 + (e ^ ((r & 3) << 2)); }
 
-// x = lo - nhi: nhi, the negated high part, exact in TF32, lo up to its last two bits.
-__device__ __forceinline__ void split_tf32(float2 x, uint32_t (&nhi)[2], uint32_t (&lo)[2]) {
-    nhi[0] = (__float_as_uint(x.x) & 0xffffe000u) ^ 0x80000000u;
-    nhi[1] = (__float_as_uint(x.y) & 0xffffe000u) ^ 0x80000000u;
-    const float2 l = add2(x, make_float2(__uint_as_float(nhi[0]), __uint_as_float(nhi[1])));
-    lo[0] = __float_as_uint(l.x);
-    lo[1] = __float_as_uint(l.y);
-}
-__device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
-                                         uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, "
-        "{%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
+// (nothing without the statistic: four CTAs of 57344 bytes fill an SM)
+template <bool ABS>
+struct AbsSums {
+    float2 h[kRows * 32];
+    __device__ __forceinline__ float2* habs() { return h; }
+};
+template <>
+struct AbsSums<false> {
+    __device__ __forceinline__ float2* habs() { return nullptr; }
+};
 
 template <bool CULL, bool ABS>
-struct BwdShared {
+struct alignas(16) BwdShared : AbsSums<ABS> {
     float4 win[kRows * 32];
-    float4 habs[ABS ? kRows * 16 : 1];
+    float4 g01[32];  // dL/dC of the lanes' two pixels, channels 0 and 1
     Stage<kSlots> st;
     float4 raw[kRing<CULL> * kChunk * 3];
 };
-
-// Monomials about the block's centre, as the B operand: entry [s][lane] holds
-// those of the two pixels that k-step s takes from lane 8 (lane % 4) + s; the
-// monomial is the lane's column lane / 4 (1, x, y, x^2, xy, y^2, 0, 0).
-struct Monomials {
-    float2 b[8][32];
-};
-__device__ __forceinline__ float monomial(int n, float x, float y) {
-    return n == 0 ? 1.0f : n == 1 ? x : n == 2 ? y : n == 3 ? x * x : n == 4 ? x * y
-           : n == 5 ? y * y : 0.0f;
-}
 
 struct BwdOut {
     float* __restrict__ grad2d;
@@ -495,90 +471,123 @@ struct BwdOut {
     float* __restrict__ partial;
 };
 
+// One sum of flush_window over the lanes of a row: x holds the pairs' sums of
+// rows {0, 1} + {4, 5}, y those of {2, 3} + {6, 7}; then the row's four lanes.
+__device__ __forceinline__ float block_sum(float2 x, float2 y) {
+    const float2 z = add2(x, y);
+    float t = __fadd_rn(z.x, z.y);
+    t = __fadd_rn(t, __shfl_xor_sync(kAll, t, 2));
+    return __fadd_rn(t, __shfl_xor_sync(kAll, t, 1));
+}
+// (scalar sums: see pair_alpha)
+__device__ __forceinline__ float2 sum2(float2 a, float2 b) {
+    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
+
 // Sums the window's rows over the block and sends the gradients of the
 // Gaussians of its first `rows` rows on their way.  slot0: the stage slot of row
-// 0.  gb: dL/dC as the B operand.
+// 0.  Lane (r, c) = (lane / 4, lane % 4) takes row r's pixel pairs of column c,
+// whose dL/dC are g01 and g2.  Every product and sum is FP32, about the Gaussian's
+// mean, in the order in which a shuffle over the lanes 16, 8, 4, 2 and 1 apart adds
+// them.
 template <int CH, bool ABS, int SLOTS>
-__device__ __forceinline__ void flush_window(const float4* win, const float4* habs,
-                                             int slot0, const Stage<SLOTS>& st,
-                                             const Monomials& mono, const uint32_t (&gb)[8][2],
-                                             int rows, float cx, float cy, const BwdOut& out) {
+__device__ __forceinline__ void flush_window(const float4* win, const float2* habs,
+                                             const float4* g01, const float2 (&g2)[kBlock],
+                                             int slot0, const Stage<SLOTS>& st, int rows, int bx,
+                                             int by, const BwdOut& out) {
     const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
     __syncwarp();
     const int slot = slot0 + r;
-    float m[4] = {0.f, 0.f, 0.f, 0.f}, k[4] = {0.f, 0.f, 0.f, 0.f};
-    float m2[4] = {0.f, 0.f, 0.f, 0.f};  // every other k-step's moments: half as long a chain of sums
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-        const float4 q = win[row_slot(r, 8 * c + s)];
-        const float2 b = mono.b[s][lane];
-        uint32_t h[2], l[2];
-        split_tf32(make_float2(q.x, q.y), h, l);
-        mma_tf32(s & 1 ? m2 : m, h[0], l[0], h[1], l[1], __float_as_uint(b.x),
-                 __float_as_uint(b.y));
-        split_tf32(make_float2(q.z, q.w), h, l);
-        mma_tf32(k, h[0], l[0], h[1], l[1], gb[s][0], gb[s][1]);
-    }
-    if constexpr (ABS) {
-        // the two magnitude sums, into columns 6 and 7
-        const uint32_t b6 = r == 6 ? __float_as_uint(1.0f) : 0u;
-        const uint32_t b7 = r == 7 ? __float_as_uint(1.0f) : 0u;
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const float4 q = habs[abs_slot(r, 4 * c + s)];
-            uint32_t h[2], l[2];
-            split_tf32(make_float2(q.x, q.z), h, l);
-            mma_tf32(m, h[0], l[0], h[1], l[1], b6, b6);
-            split_tf32(make_float2(q.y, q.w), h, l);
-            mma_tf32(m, h[0], l[0], h[1], l[1], b7, b7);
+    const float* f = reinterpret_cast<const float*>(&st.par[slot >> 1][0]) + (slot & 1);
+    const float gx = f[0], gy = f[2];
+    const float2 dx = add2(dup(gx), make_float2(-(float)(bx + 2 * c), -(float)(bx + 2 * c + 1)));
+    // the six moments (negated) and the colour weights of the pixel rows y, y + 1
+    auto two_rows = [&](int y, float2 (&m)[6], float2 (&k)[CH]) {
+        const float4 q0 = win[row_slot(r, 4 * y + c)], q1 = win[row_slot(r, 4 * y + 4 + c)];
+        const float2 t0 = mul2(make_float2(q0.x, q0.y), dx), t1 = mul2(make_float2(q1.x, q1.y), dx);
+        const float2 u0 = mul2(t0, dx), u1 = mul2(t1, dx);
+        const float2 dy = add2(dup(gy), make_float2(-(float)(by + y), -(float)(by + y + 1)));
+        m[0] = make_float2(__fadd_rn(q0.x, q0.y), __fadd_rn(q1.x, q1.y));
+        m[1] = make_float2(__fadd_rn(t0.x, t0.y), __fadd_rn(t1.x, t1.y));
+        m[2] = mul2(dy, m[0]);
+        m[3] = make_float2(__fadd_rn(u0.x, u0.y), __fadd_rn(u1.x, u1.y));
+        m[4] = mul2(dy, m[1]);
+        m[5] = mul2(dy, m[2]);
+        const float2 w0 = make_float2(q0.z, q0.w), w1 = make_float2(q1.z, q1.w);
+        if constexpr (CH == 3) {
+            const float4 a0 = g01[4 * y + c], a1 = g01[4 * y + 4 + c];
+            const float2 x0 = mul2(w0, make_float2(a0.x, a0.y)),
+                         x1 = mul2(w1, make_float2(a1.x, a1.y));
+            const float2 y0 = mul2(w0, make_float2(a0.z, a0.w)),
+                         y1 = mul2(w1, make_float2(a1.z, a1.w));
+            k[0] = make_float2(__fadd_rn(x0.x, x0.y), __fadd_rn(x1.x, x1.y));
+            k[1] = make_float2(__fadd_rn(y0.x, y0.y), __fadd_rn(y1.x, y1.y));
         }
+        const float2 z0 = mul2(w0, g2[y]), z1 = mul2(w1, g2[y + 1]);
+        k[CH - 1] = make_float2(__fadd_rn(z0.x, z0.y), __fadd_rn(z1.x, z1.y));
+    };
+    float2 m[2][6], k[2][CH];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float2 m4[6], k4[CH];
+        two_rows(2 * h, m[h], k[h]);
+        two_rows(2 * h + 4, m4, k4);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) m[h][i] = sum2(m[h][i], m4[i]);
+#pragma unroll
+        for (int i = 0; i < CH; ++i) k[h][i] = sum2(k[h][i], k4[i]);
+    }
+    float n[6], col[CH], hx = 0.0f, hy = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) n[i] = block_sum(m[0][i], m[1][i]);
+#pragma unroll
+    for (int i = 0; i < CH; ++i) col[i] = -block_sum(k[0][i], k[1][i]);
+    if constexpr (ABS) {
+        float2 p[2][2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int y = 2 * h;
+            const float2 a = habs[abs_slot(r, 4 * y + c)], b = habs[abs_slot(r, 4 * y + 4 + c)],
+                         d = habs[abs_slot(r, 4 * y + 16 + c)],
+                         e = habs[abs_slot(r, 4 * y + 20 + c)];
+            p[h][0] = sum2(make_float2(a.x, b.x), make_float2(d.x, e.x));
+            p[h][1] = sum2(make_float2(a.y, b.y), make_float2(d.y, e.y));
+        }
+        hx = block_sum(p[0][0], p[1][0]);
+        hy = block_sum(p[0][1], p[1][1]);
     }
     __syncwarp();  // the window may be written again
-    // high and low rows; the moments of row r sit in its four lanes, two each
-    const float e0 = (m[2] + m2[2]) - (m[0] + m2[0]), e1 = (m[3] + m2[3]) - (m[1] + m2[1]);
-    const float col = (k[0] - k[2]) + (k[1] - k[3]);
-    const int base = lane & ~3;
-    const float A0 = -__shfl_sync(kAll, e0, base), Sx = -__shfl_sync(kAll, e1, base);
-    const float Sy = -__shfl_sync(kAll, e0, base + 1), Sxx = -__shfl_sync(kAll, e1, base + 1);
-    const float Sxy = -__shfl_sync(kAll, e0, base + 2), Syy = -__shfl_sync(kAll, e1, base + 2);
     if (r >= rows) return;
-    const float* f = reinterpret_cast<const float*>(&st.par[slot >> 1][0]) + (slot & 1);
-    const float mx = f[0] - cx, my = f[2] - cy, nb = f[6], no = f[10];
-    const float na = 2.0f * f[4], nc = 2.0f * f[8];
+    const float nb = f[6], no = f[10], na = 2.0f * f[4], nc = 2.0f * f[8];
     constexpr int kTag = CH == 3 ? 6 : 2;
     const uint32_t id =
         __float_as_uint(reinterpret_cast<const float*>(st.col[slot])[kTag]);
-    // moments about the mean
-    const float A1 = fmaf(mx, A0, -Sx), A2 = fmaf(my, A0, -Sy);
-    const float A3 = fmaf(mx, A1 - Sx, Sxx);
-    const float A4 = fmaf(mx, A2, fmaf(-my, Sx, Sxy));
-    const float A5 = fmaf(my, A2 - Sy, Syy);
     // lane c writes components c, 4 + c (c < 2) and 6 + c (c < CH)
-    const float v0 = c == 0   ? fmaf(nb, A2, na * A1)
-                     : c == 1 ? fmaf(nb, A1, nc * A2)
-                     : c == 2 ? -0.5f * A3
-                              : -A4;
-    // A0 / o by the reciprocal and one correction of the quotient
-    const float ro = rcp_approx(no), qo = -A0 * ro;
-    const float v1 = c == 0 ? -0.5f * A5 : fmaf(fmaf(-qo, no, -A0), ro, qo);
+    const float v0 = c == 0   ? fmaf(-na, n[1], __fmul_rn(-nb, n[2]))
+                     : c == 1 ? fmaf(-nb, n[1], __fmul_rn(-nc, n[2]))
+                     : c == 2 ? 0.5f * n[3]
+                              : n[4];
+    const float v1 = c == 0 ? 0.5f * n[5] : (n[0] != 0.0f ? n[0] / no : 0.0f);
+    float v2 = col[0];
+    if constexpr (CH == 3) v2 = c == 0 ? col[0] : c == 1 ? col[1] : col[2];
     if (out.partial) {
         float* o = out.partial + (size_t)id * 11;
         o[c] = v0;
         if (c < 2) o[4 + c] = v1;
-        if (c < CH) o[6 + c] = col;
+        if (c < CH) o[6 + c] = v2;
         if (ABS && c == 3) {
-            o[9] = e0;
-            o[10] = e1;
+            o[9] = hx;
+            o[10] = hy;
         }
     } else {
         float* o = out.grad2d + (size_t)id * kGrad2d;
         if (v0 != 0.0f) atomicAdd(o + c, v0);
         if (c < 2 && v1 != 0.0f) atomicAdd(o + 4 + c, v1);
-        if (c < CH && col != 0.0f) atomicAdd(o + 6 + c, col);
+        if (c < CH && v2 != 0.0f) atomicAdd(o + 6 + c, v2);
         if (ABS && c == 3) {
             float* h = out.absgrad + (size_t)id * 2;
-            if (e0 != 0.0f) atomicAdd(h, e0);
-            if (e1 != 0.0f) atomicAdd(h + 1, e1);
+            if (hx != 0.0f) atomicAdd(h, hx);
+            if (hy != 0.0f) atomicAdd(h + 1, hy);
         }
     }
 }
@@ -626,8 +635,8 @@ __device__ __forceinline__ void adjoint_one_block(BwdPixels<CH>& s, float2 na, f
 template <int CH, bool ABS, bool HARD, int SLOTS>
 __device__ __forceinline__ void adjoint_batch(
     BwdPixels<CH>& s, const Stage<SLOTS>& st, int ns, int from0, int from1, int checked,
-    float2 nx0, float2 nx1, float2 ny, float4* win, float4* habs, const Monomials& mono,
-    const uint32_t (&gb)[8][2], float cx, float cy, const BwdOut& out) {
+    float2 nx0, float2 nx1, float2 ny, float4* win, float2* habs, const float4* g01,
+    const float2 (&g2)[kBlock], int bx, int by, const BwdOut& out) {
     const int lane = threadIdx.x & 31;
     for (int g = 0; g < ns; g += kRows) {
 #pragma unroll
@@ -662,21 +671,21 @@ __device__ __forceinline__ void adjoint_batch(
             }
             adjoint_one_block<CH, ABS>(
                 s, naA, nGA, st.col[slot], win + row_slot(2 * k, lane),
-                reinterpret_cast<float2*>(habs + abs_slot(2 * k, lane >> 1)) + (lane & 1), a.x,
+                habs + abs_slot(2 * k, lane), a.x,
                 nb.x, D.x, dx0.x, dx1.x, dy.x);
             adjoint_one_block<CH, ABS>(
                 s, naB, nGB, st.col[slot + 1], win + row_slot(2 * k + 1, lane),
-                reinterpret_cast<float2*>(habs + abs_slot(2 * k + 1, lane >> 1)) + (lane & 1), a.y,
+                habs + abs_slot(2 * k + 1, lane), a.y,
                 nb.y, D.y, dx0.y, dx1.y, dy.y);
         }
-        flush_window<CH, ABS>(win, habs, g, st, mono, gb, min(ns - g, kRows), cx, cy, out);
+        flush_window<CH, ABS>(win, habs, g01, g2, g, st, min(ns - g, kRows), bx, by, out);
     }
 }
 
 template <int CH, bool CULL, bool ABS, int SLOTS, int RING>
 __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
-                                          Feeder<SLOTS, RING>& fd, float4* win, float4* habs,
-                                          const Monomials& mono, float bg0, float bg1, float bg2,
+                                          Feeder<SLOTS, RING>& fd, float4* win, float2* habs,
+                                          float4* g01, float bg0, float bg1, float bg2,
                                           const float* __restrict__ final_T,
                                           const int32_t* __restrict__ last_idx,
                                           const float* __restrict__ dL, const BwdOut& out) {
@@ -712,27 +721,19 @@ __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
         gb2 = fma2(s.g[ch], dup(CH == 3 ? bgc[ch] : bgg), gb2);
     }
     s.nS = mul2(s.T, make_float2(-gb2.x, -gb2.y));  // minus the background seen through T_final
-    // dL/dC as the B operand: column n = lane / 4 holds the high (n even) or
-    // low part of channel n / 2
-    uint32_t gb[8][2];
+    // dL/dC of the column of pixel pairs whose sums this lane forms (flush_window):
+    // the first two channels stay in shared memory, the last one in registers
+    float2 g2[kBlock];
     {
         float2* x = reinterpret_cast<float2*>(win);
-#pragma unroll
-        for (int ch = 0; ch < CH; ++ch) x[ch * 32 + lane] = s.g[ch];
+        if constexpr (CH == 3) g01[lane] = make_float4(s.g[0].x, s.g[0].y, s.g[1].x, s.g[1].y);
+        x[lane] = s.g[CH - 1];
         __syncwarp();
-        const int n = lane >> 2, ch = n >> 1;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float2 v = ch < CH ? x[ch * 32 + 8 * (lane & 3) + k] : dup(0.0f);
-            uint32_t h[2], l[2];
-            split_tf32(v, h, l);
-            gb[k][0] = n & 1 ? l[0] : h[0] ^ 0x80000000u;
-            gb[k][1] = n & 1 ? l[1] : h[1] ^ 0x80000000u;
-        }
+        for (int y = 0; y < kBlock; ++y) g2[y] = x[4 * y + (lane & 3)];
         __syncwarp();
     }
     const float2 nx0 = dup(-(float)lx), nx1 = dup(-(float)(lx + 1)), ny = dup(-(float)ly);
-    const float cx = (float)bx + 3.5f, cy = (float)by + 3.5f;
     for (int c = 0; c < chunks;) {
         // from0, from1: the first slot of this batch within the pixel's part of the list
         int ns = 0, from0 = 0, from1 = 0;
@@ -752,15 +753,17 @@ __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
         const int checked = (int)__reduce_max_sync(kAll, (unsigned)max(from0, from1));
         if (fd.hard(ns, lane))
             adjoint_batch<CH, ABS, true>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny, win,
-                                         habs, mono, gb, cx, cy, out);
+                                       habs, g01, g2, bx, by, out);
         else
             adjoint_batch<CH, ABS, false>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny, win,
-                                          habs, mono, gb, cx, cy, out);
+                                        habs, g01, g2, bx, by, out);
         __syncwarp();  // the stage has been read
     }
     cp_async_wait_all();
     __syncwarp();
 }
+
+static_assert(sizeof(BwdShared<true, false>) * kWarps == 57344, "four CTAs per SM");
 
 template <bool CULL, bool ABS>
 __global__ void __launch_bounds__(32 * kWarps, CULL ? 4 : 5)
@@ -771,15 +774,7 @@ k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
              const float* __restrict__ final_T, const int32_t* __restrict__ last_idx,
              const float* __restrict__ dL, BwdOut out) {
     extern __shared__ float4 smem[];
-    Monomials& mono = *reinterpret_cast<Monomials*>(smem);
-    BwdShared<CULL, ABS>& my = reinterpret_cast<BwdShared<CULL, ABS>*>(
-        smem + sizeof(Monomials) / sizeof(float4))[threadIdx.x >> 5];
-    for (int i = threadIdx.x; i < 8 * 32; i += blockDim.x) {
-        const int s = i >> 5, l = i & 31, e = 8 * (l & 3) + s;
-        const float x = (float)(2 * (e & 3)) - 3.5f, y = (float)(e >> 2) - 3.5f;
-        mono.b[s][l] = make_float2(monomial(l >> 2, x, y), monomial(l >> 2, x + 1.0f, y));
-    }
-    __syncthreads();
+    BwdShared<CULL, ABS>& my = reinterpret_cast<BwdShared<CULL, ABS>*>(smem)[threadIdx.x >> 5];
     Feeder<kSlots, kRing<CULL>> fd;
     fd.raw = my.raw;
     fd.st = &my.st;
@@ -793,10 +788,10 @@ k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
         const int sub = slot & ((1 << log2_blocks) - 1);
         const int bx = (sub & ((1 << log2_bx) - 1)) * kBlock, by = (sub >> log2_bx) * kBlock;
         if (tc.channels == 3)
-            bwd_block<3, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, mono, bg0, bg1, bg2, final_T,
+            bwd_block<3, CULL, ABS>(tc, bx, by, fd, my.win, my.habs(), my.g01, bg0, bg1, bg2, final_T,
                                     last_idx, dL, out);
         else
-            bwd_block<1, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, mono, bg0, bg1, bg2, final_T,
+            bwd_block<1, CULL, ABS>(tc, bx, by, fd, my.win, my.habs(), my.g01, bg0, bg1, bg2, final_T,
                                     last_idx, dL, out);
     }
 }
@@ -865,7 +860,7 @@ gs_status launch_blocks_bwd(const Plan* p, const uint32_t* vals, void* ws, const
     const size_t per_warp =
         cull ? (abs_stats ? sizeof(BwdShared<true, true>) : sizeof(BwdShared<true, false>))
              : (abs_stats ? sizeof(BwdShared<false, true>) : sizeof(BwdShared<false, false>));
-    const size_t smem = sizeof(Monomials) + kWarps * per_warp;
+    const size_t smem = kWarps * per_warp;
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess)
