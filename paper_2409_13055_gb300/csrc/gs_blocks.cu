@@ -27,9 +27,9 @@
 // cycles per instruction each (packed FP32 runs on the heavy pipe alone), and
 // for small launches the longest list, which one warp walks.  At 1M Gaussians,
 // 1200x680, 8x8 tiles (2.0M walked (block, Gaussian) pairs), against the kernels
-// of gs_render.cu at their best launch shape: forward 182 -> 133 us, adjoint 319 ->
-// 253 us.  Sixteen views of a 500k map: 1003 -> 634 and 1593 -> 1332 us.  200k
-// Gaussians, 640x480, 16x16 tiles: 68 -> 38 and 177 -> 75 us (there the block test
+// of gs_render.cu at their best launch shape: forward 182 -> 128 us, adjoint 319 ->
+// 240 us.  Sixteen views of a 500k map: 1003 -> 629 and 1593 -> 1332 us.  200k
+// Gaussians, 640x480, 16x16 tiles: 68 -> 37 and 177 -> 74 us (there the block test
 // and the four warps per tile count as well).
 //
 // The sums on mma.sync (TF32, each operand in two parts) take 233 us at 1M but
@@ -58,6 +58,14 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 __device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+
+// A Gaussian that does not count at a pixel is multiplied by zero there.  Where a
+// colour of the map or a dL/dC of the block is wild(), the ODD variants select
+// instead.  (The projection says whether a colour is: looked for in every chunk, the
+// adjoint of 16 views of 500k took 1386 us against 1332.)
+__device__ __forceinline__ float2 where(float2 n, float2 x, float2 y) {
+    return make_float2(n.x != 0.0f ? x.x : y.x, n.y != 0.0f ? x.y : y.y);
+}
 
 // A warp's staged Gaussians.  par: pairs of slots; col: the colour, each
 // channel twice, and the slot's tag (the list position in the forward, the
@@ -97,7 +105,6 @@ struct Feeder {
     uint32_t next;         // this lane's list value of the next chunk to issue
     uint32_t tag[RING];    // ... and of the chunks in flight
     int issued;            // chunks issued so far
-    bool odd;              // some colour of the batch is not finite (forward)
 
     // pos(c): this lane's position in the list in chunk c, or -1
     template <class Pos>
@@ -154,11 +161,6 @@ struct Feeder {
 #pragma unroll
         for (int k = 1; k < RING; ++k) t = slot == k ? tag[k] : t;
         const unsigned mask = __ballot_sync(kAll, keep);
-        if (LISTPOS) {
-            const bool fin = fabsf(col.x) < INFINITY && fabsf(col.y) < INFINITY &&
-                             fabsf(col.z) < INFINITY;
-            odd = (ns > 0 && odd) || __any_sync(kAll, keep && !fin);
-        }
         issue(pos, slot, lane);
         if (keep) {
             const int s = ns + __popc(mask & ((1u << lane) - 1u));
@@ -227,7 +229,7 @@ __device__ __forceinline__ PairAlpha pair_alpha(float2 dx, float2 dy, float2 hcd
     return r;
 }
 // ... with alpha clamped at 0.99 and no weight at a positive power, for the
-// pairs that hard_pairs names (the others reach neither).
+// batches that Feeder::hard names (the others reach neither).
 __device__ __forceinline__ float2 tame(const PairAlpha& e) {
     return make_float2(e.pw.x <= 0.0f ? fmaxf(-kAlphaMax, e.noG.x) : 0.0f,
                        e.pw.y <= 0.0f ? fmaxf(-kAlphaMax, e.noG.y) : 0.0f);
@@ -246,8 +248,8 @@ struct FwdPixels {
 // Blends one Gaussian (n = -alpha where it counts at the pixel, else 0) at both
 // pixels without a branch: alpha zero leaves a pixel as it is; the Gaussian
 // that would take T below 1e-4 is not added and negates T, after which nothing
-// passes the test of Tn.
-template <int CH>
+// passes the test of Tn.  ODD: the colour may be wild.
+template <int CH, bool ODD>
 __device__ __forceinline__ void blend_one(FwdPixels<CH>& s, float2 na, const float4* col,
                                           int slot) {
     const float2 Tn = mul2(s.T, make_float2(1.0f + na.x, 1.0f + na.y));
@@ -255,11 +257,14 @@ __device__ __forceinline__ void blend_one(FwdPixels<CH>& s, float2 na, const flo
     const float2 w = mul2(na, s.T);
     const float2 nw = make_float2(a0 ? w.x : 0.0f, a1 ? w.y : 0.0f);
     const float4 c01 = col[0];
-    s.C[0] = fma2(nw, make_float2(c01.x, c01.y), s.C[0]);
+    auto add = [&](float2 c, float2& C) {
+        const float2 x = fma2(nw, c, C);
+        C = ODD ? where(nw, x, C) : x;
+    };
+    add(make_float2(c01.x, c01.y), s.C[0]);
     if constexpr (CH == 3) {
-        const float2 c2 = *reinterpret_cast<const float2*>(col + 1);
-        s.C[1] = fma2(nw, make_float2(c01.z, c01.w), s.C[1]);
-        s.C[2] = fma2(nw, c2, s.C[2]);
+        add(make_float2(c01.z, c01.w), s.C[1]);
+        add(*reinterpret_cast<const float2*>(col + 1), s.C[2]);
     }
     s.l0 = nw.x < 0.0f ? slot : s.l0;
     s.l1 = nw.y < 0.0f ? slot : s.l1;
@@ -267,12 +272,12 @@ __device__ __forceinline__ void blend_one(FwdPixels<CH>& s, float2 na, const flo
     s.T.y = a1 ? Tn.y : -fabsf(s.T.y);
 }
 
-// Blends a staged batch.  HARD: alphas are clamped, positive powers skipped and
-// (odd) the two Gaussians of a pair voted on apart, so that a colour that is
-// not finite stays with the blocks that blend it.
-template <int CH, bool HARD, int SLOTS>
+// Blends a staged batch.  HARD: alphas are clamped and positive powers skipped.
+// ODD: some colour is wild.
+template <int CH, bool HARD, bool ODD, int SLOTS>
 __device__ __forceinline__ void blend_batch(FwdPixels<CH>& s, const Stage<SLOTS>& st, int ns,
-                                            float2 nx0, float2 nx1, float2 ny, bool odd) {
+                                            float2 nx0, float2 nx1, float2 ny) {
+    constexpr int kS = ODD ? 1 : kStep;
     auto evaluate = [&](int p, float2& n0, float2& n1) {
         const float4 A = st.par[p][0], B = st.par[p][1], D = st.par[p][2];
         const float2 dy = add2(make_float2(A.z, A.w), ny);
@@ -284,11 +289,11 @@ __device__ __forceinline__ void blend_batch(FwdPixels<CH>& s, const Stage<SLOTS>
         n0 = HARD ? tame(e0) : e0.noG;
         n1 = HARD ? tame(e1) : e1.noG;
     };
-    for (int p = 0; 2 * p < ns; p += kStep) {
-        float2 n0[kStep], n1[kStep];
+    for (int p = 0; 2 * p < ns; p += kS) {
+        float2 n0[kS], n1[kS];
         bool mine0 = false, mine1 = false;
 #pragma unroll
-        for (int k = 0; k < kStep; ++k) {
+        for (int k = 0; k < kS; ++k) {
             evaluate(p + k, n0[k], n1[k]);
             mine0 = mine0 || fminf(n0[k].x, n0[k].y) <= -kAlphaMin;
             mine1 = mine1 || fminf(n1[k].x, n1[k].y) <= -kAlphaMin;
@@ -299,16 +304,14 @@ __device__ __forceinline__ void blend_batch(FwdPixels<CH>& s, const Stage<SLOTS>
             continue;
         }
 #pragma unroll
-        for (int k = 0; k < kStep; ++k) {
+        for (int k = 0; k < kS; ++k) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const float a0 = h ? n0[k].y : n0[k].x, a1 = h ? n1[k].y : n1[k].x;
-                const bool h0 = a0 <= -kAlphaMin, h1 = a1 <= -kAlphaMin;
-                if (HARD && odd &&
-                    !__any_sync(kAll, (h0 && s.T.x > 0.0f) || (h1 && s.T.y > 0.0f)))
-                    continue;
-                blend_one<CH>(s, make_float2(h0 ? a0 : 0.0f, h1 ? a1 : 0.0f),
-                              st.col[2 * (p + k) + h], 2 * (p + k) + h);
+                const float2 na = make_float2(a0 <= -kAlphaMin ? a0 : 0.0f,
+                                              a1 <= -kAlphaMin ? a1 : 0.0f);
+                const int slot = 2 * (p + k) + h;
+                blend_one<CH, ODD>(s, na, st.col[slot], slot);
             }
         }
     }
@@ -316,8 +319,9 @@ __device__ __forceinline__ void blend_batch(FwdPixels<CH>& s, const Stage<SLOTS>
 
 template <int CH, bool CULL, int SLOTS, int RING>
 __device__ __forceinline__ void fwd_block(const ViewTable& vt, const TileCtx& tc, int bx, int by,
-                                          Feeder<SLOTS, RING>& fd, float bg0, float bg1, float bg2,
-                                          float* __restrict__ images, float* __restrict__ final_T,
+                                          Feeder<SLOTS, RING>& fd, bool odd, float bg0, float bg1,
+                                          float bg2, float* __restrict__ images,
+                                          float* __restrict__ final_T,
                                           int32_t* __restrict__ last_idx) {
     const int lane = threadIdx.x & 31;
     const int lx = bx + 2 * (lane & 3), ly = by + (lane >> 2);
@@ -349,10 +353,12 @@ __device__ __forceinline__ void fwd_block(const ViewTable& vt, const TileCtx& tc
         fd.template pad<2 * kStep>(ns, lane);
         __syncwarp();
         s.l0 = s.l1 = -1;
-        if (fd.hard(ns, lane) || fd.odd)
-            blend_batch<CH, true>(s, *fd.st, ns, nx0, nx1, ny, fd.odd);
+        if (odd)
+            blend_batch<CH, true, true>(s, *fd.st, ns, nx0, nx1, ny);
+        else if (fd.hard(ns, lane))
+            blend_batch<CH, true, false>(s, *fd.st, ns, nx0, nx1, ny);
         else
-            blend_batch<CH, false>(s, *fd.st, ns, nx0, nx1, ny, false);
+            blend_batch<CH, false, false>(s, *fd.st, ns, nx0, nx1, ny);
         constexpr int kTag = CH == 3 ? 6 : 2;
         if (s.l0 >= 0)
             last0 = __float_as_int(reinterpret_cast<const float*>(fd.st->col[s.l0])[kTag]) + 1;
@@ -409,7 +415,8 @@ __global__ void __launch_bounds__(32 * kWarps, CULL ? 5 : 8)
 k_blocks_fwd(ViewTable vt, const uint32_t* __restrict__ ranges,
              const uint32_t* __restrict__ order, const uint32_t* __restrict__ ivals,
              const uint32_t* __restrict__ gid_of, const float4* __restrict__ rec, int log2_bx,
-             int log2_blocks, int total_blocks, uint32_t* queue, float bg0, float bg1, float bg2,
+             int log2_blocks, int total_blocks, uint32_t* queue,
+             const DevCounters* __restrict__ ctr, float bg0, float bg1, float bg2,
              float* __restrict__ images, float* __restrict__ final_T,
              int32_t* __restrict__ last_idx) {
     __shared__ FwdShared<CULL> sh[kWarps];
@@ -420,6 +427,7 @@ k_blocks_fwd(ViewTable vt, const uint32_t* __restrict__ ranges,
     fd.ivals = ivals;
     fd.gid_of = gid_of;
     fd.rec = rec;
+    const bool wild_map = ctr->wild_colour != 0u;
     for (;;) {
         const int slot = next_slot(queue);
         if (slot >= total_blocks) break;
@@ -428,9 +436,11 @@ k_blocks_fwd(ViewTable vt, const uint32_t* __restrict__ ranges,
         const int bx = (sub & ((1 << log2_bx) - 1)) * kBlock, by = (sub >> log2_bx) * kBlock;
         if (tc.tx0 + bx >= tc.width || tc.ty0 + by >= tc.height) continue;
         if (tc.channels == 3)
-            fwd_block<3, CULL>(vt, tc, bx, by, fd, bg0, bg1, bg2, images, final_T, last_idx);
+            fwd_block<3, CULL>(vt, tc, bx, by, fd, wild_map, bg0, bg1, bg2, images, final_T,
+                               last_idx);
         else
-            fwd_block<1, CULL>(vt, tc, bx, by, fd, bg0, bg1, bg2, images, final_T, last_idx);
+            fwd_block<1, CULL>(vt, tc, bx, by, fd, wild_map, bg0, bg1, bg2, images, final_T,
+                               last_idx);
     }
 }
 
@@ -446,21 +456,12 @@ __device__ __forceinline__ int row_slot(int r, int e) { return r * 32 + (e ^ ((r
 // ... and {|h_x|, |h_y|} of the density statistic.
 __device__ __forceinline__ int abs_slot(int r, int e) { return r * 32 + (e ^ ((r & 3) << 2)); }
 
-// (nothing without the statistic: four CTAs of 57344 bytes fill an SM)
-template <bool ABS>
-struct AbsSums {
-    float2 h[kRows * 32];
-    __device__ __forceinline__ float2* habs() { return h; }
-};
-template <>
-struct AbsSums<false> {
-    __device__ __forceinline__ float2* habs() { return nullptr; }
-};
-
 template <bool CULL, bool ABS>
-struct alignas(16) BwdShared : AbsSums<ABS> {
+struct BwdShared {
     float4 win[kRows * 32];
+    float2 habs[ABS ? kRows * 32 : 2];
     float4 g01[32];  // dL/dC of the lanes' two pixels, channels 0 and 1
+    float2 g2[32];   // ... and the last channel
     Stage<kSlots> st;
     float4 raw[kRing<CULL> * kChunk * 3];
 };
@@ -489,10 +490,10 @@ __device__ __forceinline__ float2 sum2(float2 a, float2 b) {
 // 0.  Lane (r, c) = (lane / 4, lane % 4) takes row r's pixel pairs of column c,
 // whose dL/dC are g01 and g2.  Every product and sum is FP32, about the Gaussian's
 // mean, in the order in which a shuffle over the lanes 16, 8, 4, 2 and 1 apart adds
-// them.
-template <int CH, bool ABS, int SLOTS>
+// them.  ODD: colours or dL/dC may be wild().
+template <int CH, bool ABS, bool ODD, int SLOTS>
 __device__ __forceinline__ void flush_window(const float4* win, const float2* habs,
-                                             const float4* g01, const float2 (&g2)[kBlock],
+                                             const float4* g01, const float2* g2,
                                              int slot0, const Stage<SLOTS>& st, int rows, int bx,
                                              int by, const BwdOut& out) {
     const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
@@ -514,16 +515,20 @@ __device__ __forceinline__ void flush_window(const float4* win, const float2* ha
         m[4] = mul2(dy, m[1]);
         m[5] = mul2(dy, m[2]);
         const float2 w0 = make_float2(q0.z, q0.w), w1 = make_float2(q1.z, q1.w);
+        auto weigh = [](float2 w, float2 g) {
+            const float2 x = mul2(w, g);
+            return ODD ? where(w, x, dup(0.0f)) : x;
+        };
         if constexpr (CH == 3) {
             const float4 a0 = g01[4 * y + c], a1 = g01[4 * y + 4 + c];
-            const float2 x0 = mul2(w0, make_float2(a0.x, a0.y)),
-                         x1 = mul2(w1, make_float2(a1.x, a1.y));
-            const float2 y0 = mul2(w0, make_float2(a0.z, a0.w)),
-                         y1 = mul2(w1, make_float2(a1.z, a1.w));
+            const float2 x0 = weigh(w0, make_float2(a0.x, a0.y)),
+                         x1 = weigh(w1, make_float2(a1.x, a1.y));
+            const float2 y0 = weigh(w0, make_float2(a0.z, a0.w)),
+                         y1 = weigh(w1, make_float2(a1.z, a1.w));
             k[0] = make_float2(__fadd_rn(x0.x, x0.y), __fadd_rn(x1.x, x1.y));
             k[1] = make_float2(__fadd_rn(y0.x, y0.y), __fadd_rn(y1.x, y1.y));
         }
-        const float2 z0 = mul2(w0, g2[y]), z1 = mul2(w1, g2[y + 1]);
+        const float2 z0 = weigh(w0, g2[4 * y + c]), z1 = weigh(w1, g2[4 * y + 4 + c]);
         k[CH - 1] = make_float2(__fadd_rn(z0.x, z0.y), __fadd_rn(z1.x, z1.y));
     };
     float2 m[2][6], k[2][CH];
@@ -600,8 +605,9 @@ struct BwdPixels {
 // One Gaussian's adjoint at the lane's two pixels into a row of the window
 // (win, habs: the lane's places in it).  na: -alpha where the Gaussian counts
 // at the pixel, else 0, which leaves the pixel's state as it is; nG: -o G where
-// alpha = o G, 0 where alpha is clamped (and passes no gradient).
-template <int CH, bool ABS>
+// alpha = o G, 0 where alpha is clamped (and passes no gradient).  ODD: the colour or
+// dL/dC may be wild.
+template <int CH, bool ABS, bool ODD>
 __device__ __forceinline__ void adjoint_one_block(BwdPixels<CH>& s, float2 na, float2 nG,
                                                   const float4* col, float4* win, float2* habs,
                                                   float ha, float nb, float hc, float dx0,
@@ -617,8 +623,10 @@ __device__ __forceinline__ void adjoint_one_block(BwdPixels<CH>& s, float2 na, f
         gc = fma2(s.g[2], c2, gc);
     }
     const float2 dal = fma2(s.T, gc, mul2(inv, s.nS));
-    s.nS = fma2(nw, gc, s.nS);
-    const float2 ndp = mul2(nG, dal);
+    const float2 nS = fma2(nw, gc, s.nS);
+    s.nS = ODD ? where(na, nS, s.nS) : nS;
+    float2 ndp = mul2(nG, dal);
+    if (ODD) ndp = where(nG, ndp, dup(0.0f));
     *win = make_float4(ndp.x, ndp.y, nw.x, nw.y);
     if constexpr (ABS) {
         // each pixel's own contribution to dL/dmean2d, by magnitude
@@ -631,15 +639,16 @@ __device__ __forceinline__ void adjoint_one_block(BwdPixels<CH>& s, float2 na, f
 
 // The adjoint of a staged batch, eight slots (a window) at a time.  Every slot
 // takes its row: nearly all reach a pixel of the block, and a row of zeros costs
-// less than finding out.  HARD: alphas are clamped and positive powers skipped.
-template <int CH, bool ABS, bool HARD, int SLOTS>
+// less than finding out.  HARD: alphas are clamped and positive powers skipped; ODD:
+// colours or dL/dC may be wild.
+template <int CH, bool ABS, bool HARD, bool ODD, int SLOTS>
 __device__ __forceinline__ void adjoint_batch(
     BwdPixels<CH>& s, const Stage<SLOTS>& st, int ns, int from0, int from1, int checked,
     float2 nx0, float2 nx1, float2 ny, float4* win, float2* habs, const float4* g01,
-    const float2 (&g2)[kBlock], int bx, int by, const BwdOut& out) {
+    const float2* g2, int bx, int by, const BwdOut& out) {
     const int lane = threadIdx.x & 31;
     for (int g = 0; g < ns; g += kRows) {
-#pragma unroll
+#pragma unroll(ODD ? 1 : kRows / 2)
         for (int k = 0; k < kRows / 2; ++k) {
             const int slot = g + 2 * k;
             const float4 A = st.par[slot >> 1][0], B = st.par[slot >> 1][1],
@@ -669,23 +678,24 @@ __device__ __forceinline__ void adjoint_batch(
                 nGB = make_float2(e0.noG.y > -kAlphaMax ? naB.x : 0.0f,
                                   e1.noG.y > -kAlphaMax ? naB.y : 0.0f);
             }
-            adjoint_one_block<CH, ABS>(
+            adjoint_one_block<CH, ABS, ODD>(
                 s, naA, nGA, st.col[slot], win + row_slot(2 * k, lane),
                 habs + abs_slot(2 * k, lane), a.x,
                 nb.x, D.x, dx0.x, dx1.x, dy.x);
-            adjoint_one_block<CH, ABS>(
+            adjoint_one_block<CH, ABS, ODD>(
                 s, naB, nGB, st.col[slot + 1], win + row_slot(2 * k + 1, lane),
                 habs + abs_slot(2 * k + 1, lane), a.y,
                 nb.y, D.y, dx0.y, dx1.y, dy.y);
         }
-        flush_window<CH, ABS>(win, habs, g01, g2, g, st, min(ns - g, kRows), bx, by, out);
+        flush_window<CH, ABS, ODD>(win, habs, g01, g2, g, st, min(ns - g, kRows), bx, by, out);
     }
 }
 
 template <int CH, bool CULL, bool ABS, int SLOTS, int RING>
 __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
                                           Feeder<SLOTS, RING>& fd, float4* win, float2* habs,
-                                          float4* g01, float bg0, float bg1, float bg2,
+                                          float4* g01, float2* g2, bool wild_map, float bg0,
+                                          float bg1, float bg2,
                                           const float* __restrict__ final_T,
                                           const int32_t* __restrict__ last_idx,
                                           const float* __restrict__ dL, const BwdOut& out) {
@@ -714,25 +724,21 @@ __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
     const float bgc[3] = {bg0, bg1, bg2};
     const float bgg = (bg0 + bg1 + bg2) * (1.0f / 3.0f);
     float2 gb2 = dup(0.0f);
+    bool big = false;
 #pragma unroll
     for (int ch = 0; ch < CH; ++ch) {
         const float* d = dL + tc.val_base + ch * plane + pix;
         s.g[ch] = make_float2(in0 ? d[0] : 0.0f, in1 ? d[1] : 0.0f);
+        big = big || wild(s.g[ch].x) || wild(s.g[ch].y);
         gb2 = fma2(s.g[ch], dup(CH == 3 ? bgc[ch] : bgg), gb2);
     }
+    const bool odd = __any_sync(kAll, big) || wild_map;
     s.nS = mul2(s.T, make_float2(-gb2.x, -gb2.y));  // minus the background seen through T_final
-    // dL/dC of the column of pixel pairs whose sums this lane forms (flush_window):
-    // the first two channels stay in shared memory, the last one in registers
-    float2 g2[kBlock];
-    {
-        float2* x = reinterpret_cast<float2*>(win);
-        if constexpr (CH == 3) g01[lane] = make_float4(s.g[0].x, s.g[0].y, s.g[1].x, s.g[1].y);
-        x[lane] = s.g[CH - 1];
-        __syncwarp();
-#pragma unroll
-        for (int y = 0; y < kBlock; ++y) g2[y] = x[4 * y + (lane & 3)];
-        __syncwarp();
-    }
+    // for flush_window (as registers of the lanes that need them: 251 us at 1M
+    // against 239)
+    if constexpr (CH == 3) g01[lane] = make_float4(s.g[0].x, s.g[0].y, s.g[1].x, s.g[1].y);
+    g2[lane] = s.g[CH - 1];
+    __syncwarp();
     const float2 nx0 = dup(-(float)lx), nx1 = dup(-(float)(lx + 1)), ny = dup(-(float)ly);
     for (int c = 0; c < chunks;) {
         // from0, from1: the first slot of this batch within the pixel's part of the list
@@ -751,26 +757,29 @@ __device__ __forceinline__ void bwd_block(const TileCtx& tc, int bx, int by,
         __syncwarp();
         // slots before this one may lie beyond some pixel's part of the list
         const int checked = (int)__reduce_max_sync(kAll, (unsigned)max(from0, from1));
-        if (fd.hard(ns, lane))
-            adjoint_batch<CH, ABS, true>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny, win,
-                                       habs, g01, g2, bx, by, out);
+        if (odd)
+            adjoint_batch<CH, ABS, true, true>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny,
+                                               win, habs, g01, g2, bx, by, out);
+        else if (fd.hard(ns, lane))
+            adjoint_batch<CH, ABS, true, false>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny,
+                                                win, habs, g01, g2, bx, by, out);
         else
-            adjoint_batch<CH, ABS, false>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny, win,
-                                        habs, g01, g2, bx, by, out);
+            adjoint_batch<CH, ABS, false, false>(s, *fd.st, ns, from0, from1, checked, nx0, nx1, ny,
+                                                 win, habs, g01, g2, bx, by, out);
         __syncwarp();  // the stage has been read
     }
     cp_async_wait_all();
     __syncwarp();
 }
 
-static_assert(sizeof(BwdShared<true, false>) * kWarps == 57344, "four CTAs per SM");
 
 template <bool CULL, bool ABS>
 __global__ void __launch_bounds__(32 * kWarps, CULL ? 4 : 5)
 k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
              const uint32_t* __restrict__ order, const uint32_t* __restrict__ ivals,
              const uint32_t* __restrict__ gid_of, const float4* __restrict__ rec, int log2_bx,
-             int log2_blocks, int total_blocks, uint32_t* queue, float bg0, float bg1, float bg2,
+             int log2_blocks, int total_blocks, uint32_t* queue,
+             const DevCounters* __restrict__ ctr, float bg0, float bg1, float bg2,
              const float* __restrict__ final_T, const int32_t* __restrict__ last_idx,
              const float* __restrict__ dL, BwdOut out) {
     extern __shared__ float4 smem[];
@@ -781,6 +790,7 @@ k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
     fd.ivals = ivals;
     fd.gid_of = gid_of;
     fd.rec = rec;
+    const bool wild_map = ctr->wild_colour != 0u;
     for (;;) {
         const int slot = next_slot(queue);
         if (slot >= total_blocks) break;
@@ -788,11 +798,11 @@ k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
         const int sub = slot & ((1 << log2_blocks) - 1);
         const int bx = (sub & ((1 << log2_bx) - 1)) * kBlock, by = (sub >> log2_bx) * kBlock;
         if (tc.channels == 3)
-            bwd_block<3, CULL, ABS>(tc, bx, by, fd, my.win, my.habs(), my.g01, bg0, bg1, bg2, final_T,
-                                    last_idx, dL, out);
+            bwd_block<3, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, my.g01, my.g2, wild_map, bg0,
+                                    bg1, bg2, final_T, last_idx, dL, out);
         else
-            bwd_block<1, CULL, ABS>(tc, bx, by, fd, my.win, my.habs(), my.g01, bg0, bg1, bg2, final_T,
-                                    last_idx, dL, out);
+            bwd_block<1, CULL, ABS>(tc, bx, by, fd, my.win, my.habs, my.g01, my.g2, wild_map, bg0,
+                                    bg1, bg2, final_T, last_idx, dL, out);
     }
 }
 
@@ -843,8 +853,9 @@ gs_status launch_blocks_fwd(const Plan* p, const uint32_t* vals, void* ws, float
     kern<<<blocks, 32 * kWarps, 0, st>>>(
         p->vt, cbuf<uint32_t>(p, ws, GS_BUF_RANGES), cbuf<uint32_t>(p, ws, B_TILE_ORDER), vals,
         p->cfg.deterministic ? cbuf<uint32_t>(p, ws, B_GID_OF) : nullptr,
-        cbuf<float4>(p, ws, GS_BUF_PROJ), log2_bx, log2_blocks, total, queue, p->cfg.bg[0],
-        p->cfg.bg[1], p->cfg.bg[2], images, final_T, last_idx);
+        cbuf<float4>(p, ws, GS_BUF_PROJ), log2_bx, log2_blocks, total, queue,
+        cbuf<DevCounters>(p, ws, GS_BUF_COUNTERS), p->cfg.bg[0], p->cfg.bg[1], p->cfg.bg[2],
+        images, final_T, last_idx);
     return launch_status();
 }
 
@@ -876,8 +887,9 @@ gs_status launch_blocks_bwd(const Plan* p, const uint32_t* vals, void* ws, const
     kern<<<blocks, 32 * kWarps, smem, st>>>(
         p->vt, cbuf<uint32_t>(p, ws, GS_BUF_RANGES), cbuf<uint32_t>(p, ws, B_TILE_ORDER), vals,
         p->cfg.deterministic ? cbuf<uint32_t>(p, ws, B_GID_OF) : nullptr,
-        cbuf<float4>(p, ws, GS_BUF_PROJ), log2_bx, log2_blocks, total, queue, p->cfg.bg[0],
-        p->cfg.bg[1], p->cfg.bg[2], final_T, last_idx, dL, out);
+        cbuf<float4>(p, ws, GS_BUF_PROJ), log2_bx, log2_blocks, total, queue,
+        cbuf<DevCounters>(p, ws, GS_BUF_COUNTERS), p->cfg.bg[0], p->cfg.bg[1], p->cfg.bg[2],
+        final_T, last_idx, dL, out);
     return launch_status();
 }
 

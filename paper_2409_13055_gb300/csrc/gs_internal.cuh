@@ -122,7 +122,12 @@ struct DevCounters {
     uint32_t n_sorted;             // visible pairs kept by the first depth pass
     uint32_t span_pool_used;       // rows of B_SPAN_POOL taken by the last gs_project
     uint32_t max_key;              // largest depth key of its visible pairs
+    uint32_t wild_colour;          // 1: one of them has a colour that is wild()
 };
+
+// Colours and dL/dC whose products may not be finite: the render kernels over blocks
+// (gs_blocks.cu) then select where they otherwise multiply by zero.
+__device__ __forceinline__ bool wild(float x) { return !(fabsf(x) < 1e15f); }
 
 static_assert(offsetof(DevCounters, status) == 0, "gs_project keeps the leading status word");
 

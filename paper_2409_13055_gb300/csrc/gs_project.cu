@@ -498,6 +498,8 @@ k_project(const float* __restrict__ means, const float* __restrict__ log_scales,
         }
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) col[ch] = fmaxf(col[ch] + 0.5f, 0.0f);
+        // (no colour is below zero or NaN)
+        if (wild(fmaxf(fmaxf(col[0], col[1]), col[2]))) counters->wild_colour = 1u;
         float4* r = rec + vg * 3;
         r[0] = make_float4(p.mxh, p.myh, p.mxl, p.myl);
         r[1] = make_float4(p.ca, p.cb, p.cc, opacity);
