@@ -77,10 +77,12 @@ struct Stage {
 };
 
 // Whether the Gaussian's alpha can reach 1/255 in the pixels [x0, x0 + 7] x
-// [y0, y0 + 7]: q(d) = a dx^2 + 2 b dx dy + c dy^2 against 2 ln(255 o), the
-// level widened by 1% + 0.02, far beyond the rounding of either side.  The
+// [y0, y0 + 7]: q(d) = a dx^2 + 2 b dx dy + c dy^2 against 2 ln(255 o).  The
 // smallest q over a rectangle that does not hold the mean lies on one of the
-// two edges that face it.
+// two edges that face it.  The level is widened by what rounding can do: 1% +
+// 0.02 for the logarithm and the exponential, and for the form's terms, which
+// cancel along a needle, 2e-6 of the largest sum of their magnitudes in the block
+// (a pixel's power and q here are each off by at most six roundings of 2^-24 of it).
 __device__ __forceinline__ bool meets_block(float lx, float ly, float a, float b, float c,
                                             float o, float x0, float y0) {
     const float xe = fminf(fmaxf(lx, x0), x0 + 7.0f) - lx;
@@ -89,7 +91,9 @@ __device__ __forceinline__ bool meets_block(float lx, float ly, float a, float b
     const float dx = fminf(fmaxf(__fdividef(-b * ye, a), x0 - lx), x0 + 7.0f - lx);
     const float q1 = fmaf(a * xe, xe, fmaf(2.0f * b * xe, dy, c * dy * dy));
     const float q2 = fmaf(a * dx, dx, fmaf(2.0f * b * dx, ye, c * ye * ye));
-    const float level = 2.02f * __logf(255.0f * o) + 0.02f;
+    const float X = fabsf(x0 + 3.5f - lx) + 3.5f, Y = fabsf(y0 + 3.5f - ly) + 3.5f;
+    const float most = fmaf(a * X, X, fmaf(2.0f * fabsf(b) * X, Y, c * Y * Y));
+    const float level = fmaf(2e-6f, most, 2.02f * __logf(255.0f * o) + 0.02f);
     return !(fminf(q1, q2) > level);
 }
 
