@@ -128,7 +128,8 @@ __device__ __forceinline__ void issue_batch(const TM& tm, float4* stage, uint32_
 // Replace the mean pair of each staged record by its tile-local offset:
 // stage[3j] = {lx, ly, a, b}; stage[3j+1] = {a, b, c, o}; stage[3j+2] =
 // {r, g, b, gray}; and record in wmask[j] which warps of the CTA the Gaussian
-// can reach.  Warp w owns tile rows [w*rows, (w+1)*rows).  A warp is left out
+// can reach.  Warp w owns `per` pixels from w*per on, row by row: whole rows, or part
+// of one row of a tile wider than that (whose strip is the row).  A warp is left out
 // only if its pixel strip misses the bounding box of the Gaussian's
 // alpha >= 1/255 ellipse, {d : d^T Q d <= 2 ln(255 o)}, whose half-extents
 // are sqrt(2 ln(255 o) (Q^-1)_xx) and sqrt(2 ln(255 o) (Q^-1)_yy); the box is
@@ -141,8 +142,9 @@ __device__ __forceinline__ void issue_batch(const TM& tm, float4* stage, uint32_
 // Gaussian is evaluated and the alpha test decides.
 template <class TM>
 __device__ __forceinline__ void localise_batch(const TM& tm, float4* stage, uint32_t* wmask,
-                                               int cnt, float tx0, float ty0, int tile_w, int rows,
-                                               int nwarps, bool masks = true) {
+                                               int cnt, float tx0, float ty0, int log2_tw,
+                                               int per, int nwarps, bool masks = true) {
+    const int tile_w = 1 << log2_tw;
     for (int j = tm.tid; j < cnt; j += tm.size) {
         float4 m = stage[3 * j];
         const float4 q = stage[3 * j + 1];
@@ -169,7 +171,8 @@ __device__ __forceinline__ void localise_batch(const TM& tm, float4* stage, uint
                     bits = all;
                 } else if (m.x + ex >= 0.0f && m.x - ex <= (float)(tile_w - 1)) {
                     for (int w = 0; w < nwarps; ++w) {
-                        const float r0 = (float)(w * rows), r1 = (float)(w * rows + rows - 1);
+                        const float r0 = (float)((w * per) >> log2_tw);
+                        const float r1 = (float)(((w + 1) * per - 1) >> log2_tw);
                         if (m.y + ey >= r0 && m.y - ey <= r1) bits |= 1u << w;
                     }
                 }
@@ -365,7 +368,6 @@ __device__ void render_fwd_tile(const TM& tm, const ViewTable& vt, const TileCtx
                                 float* __restrict__ final_T, int32_t* __restrict__ last_idx) {
     uint32_t* const mask0 = reinterpret_cast<uint32_t*>(smem + 6 * batch);
     const int nwarps = tm.size >> 5;
-    const int rows = (32 * PPT) >> vt.log2_tw;
     const PixelRun pr = pixel_run(tm.tid, PPT, vt.log2_tw, vt.tile_w);
     const int py = tc.ty0 + pr.ly;
     // per-warp culling only where a warp covers part of the tile or the
@@ -407,8 +409,8 @@ __device__ void render_fwd_tile(const TM& tm, const ViewTable& vt, const TileCtx
         }
         tm.sync();
         uint32_t* cmask = mask0 + (b & 1) * batch;
-        localise_batch(tm, cur, cmask, cnt, (float)tc.tx0, (float)tc.ty0, vt.tile_w, rows, nwarps,
-                       cull);
+        localise_batch(tm, cur, cmask, cnt, (float)tc.tx0, (float)tc.ty0, vt.log2_tw, 32 * PPT,
+                       nwarps, cull);
         tm.sync();
         blend_batch<CH, PPT>(tm.tid, cur, cmask, cnt, (uint32_t)(b * batch), pr.lx0,
                              (float)pr.ly, T, C, last, live, nlx, cull);
@@ -653,7 +655,6 @@ __device__ void render_bwd_tile(const TM& tm, const ViewTable& vt, const TileCtx
     uint32_t* const mask0 = ids0 + 2 * batch;
     float* const acc = reinterpret_cast<float*>(mask0 + 2 * batch);
     const int nwarps = tm.size >> 5;
-    const int rows = (32 * PPT) >> vt.log2_tw;
     const uint32_t wbit = 1u << (tm.tid >> 5);
     // per-warp culling only where a warp covers part of the tile or the
     // tile lists are the square rects
@@ -729,8 +730,8 @@ __device__ void render_bwd_tile(const TM& tm, const ViewTable& vt, const TileCtx
             cp_async_wait_all();
         }
         tm.sync();
-        localise_batch(tm, cur, cmask, cnt, (float)tc.tx0, (float)tc.ty0, vt.tile_w, rows, nwarps,
-                       cull);
+        localise_batch(tm, cur, cmask, cnt, (float)tc.tx0, (float)tc.ty0, vt.log2_tw, 32 * PPT,
+                       nwarps, cull);
         tm.sync();
         if constexpr (PPT % 2 == 0) {
             // one Gaussian, its values reduced alone
