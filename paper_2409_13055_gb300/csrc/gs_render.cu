@@ -133,8 +133,11 @@ __device__ __forceinline__ void issue_batch(const TM& tm, float4* stage, uint32_
 // only if its pixel strip misses the bounding box of the Gaussian's
 // alpha >= 1/255 ellipse, {d : d^T Q d <= 2 ln(255 o)}, whose half-extents
 // are sqrt(2 ln(255 o) (Q^-1)_xx) and sqrt(2 ln(255 o) (Q^-1)_yy); the box is
-// grown by 0.1% + 0.01 px, far beyond FP32 rounding, so every skipped
-// evaluation would have been skipped by the alpha test itself.
+// grown by 0.1% + 0.01 px, beyond FP32 rounding where the conic is not a long
+// needle's: with det Q >= 1e-3 a c the determinant is off by at most 2e-4 of itself
+// and a pixel's form by 0.016, so every skipped evaluation would have been
+// skipped by the alpha test itself.  Longer needles (63 to 1 and beyond) are left
+// out of no warp.
 // With masks false the warp masks are neither formed nor written: for a team
 // of one warp over tight tile sets, whose listed Gaussians all reach the
 // tile's ellipse box up to the margins, the mask would leave the warp out of
@@ -162,7 +165,7 @@ __device__ __forceinline__ void localise_batch(const TM& tm, float4* stage, uint
         const float tau = logf(255.0f * q.w);
         const float detq = q.x * q.z - q.y * q.y;
         if (tau > 0.0f) {
-            if (!(detq > 0.0f)) {
+            if (!(detq > 1e-3f * (q.x * q.z))) {
                 bits = all;
             } else {
                 const float ex = sqrtf(2.0f * tau * q.z / detq) * 1.001f + 0.01f;

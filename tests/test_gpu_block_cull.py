@@ -40,6 +40,30 @@ def _needles(rng, n, sigma, reach, f=600.0, z=2.0):
                 sh=rng.uniform(-1, 1, (1, n, 3)).astype(np.float32), sh_degree=0)
 
 
+NEEDLES = [(30, 60), (100, 200), (800, 1500), (3000, 700), (3000, 5000), (20000, 16000)]
+
+
+@pytest.mark.parametrize("sigma,reach", NEEDLES)
+@pytest.mark.parametrize("kw", [dict(pixels_per_thread_bwd=8),
+                                dict(pixels_per_thread=2, pixels_per_thread_bwd=8),
+                                dict(pixels_per_thread=8, tight_rect=False)])
+def test_tile_kernels_leave_no_needle_out_either(sigma, reach, kw):
+    """The masks of the tile kernels' warps: the bits of the block kernels."""
+    rng = np.random.default_rng(sigma)
+    p = _needles(rng, 300, sigma, reach)
+    view = scenes.camera(1200, 680, 600.0, 600.0)
+    gm = mapping.GaussianMap(p)
+    out = []
+    for k in (dict(tight_rect=kw.get("tight_rect", True)), dict(kw, deterministic=True)):
+        rast = mapping.Rasterizer([view], gm.n, instance_capacity=1 << 20, **k)
+        rast.forward(gm.gs_map())
+        torch.cuda.synchronize()
+        assert rast.counters().status == 0
+        out.append([t.cpu().numpy() for t in (rast.images, rast.final_T, rast.last_idx)])
+    for x, y in zip(*out):
+        np.testing.assert_array_equal(x, y)
+
+
 @pytest.mark.parametrize("sigma,reach", [(100, 200), (800, 1500), (3000, 700), (3000, 5000),
                                          (20000, 16000)])
 def test_long_needles_are_in_every_block_they_reach(sigma, reach):
