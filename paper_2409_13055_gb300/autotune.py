@@ -1,18 +1,18 @@
 """Autotuner for the rasteriser's launch shape.
 
-Picks the tile shape (8x8, 16x16, 32x8), then the number of Gaussians staged
-per shared-memory batch and the pixels per thread separately for the forward
-and the backward kernel, by timing the projection, binning, forward, loss and
-backward of one mapping iteration on the caller's own map and views with CUDA
-events (Adam is independent of these choices and is left out, so the map is
-not modified).
+Picks the tile shape (8x8, 16x16, 32x8) by timing the projection, binning,
+forward, loss and backward of one mapping iteration on the caller's own map and
+views with CUDA events (Adam is independent of the choice and is left out, so
+the map is not modified).  These tiles are whole 8x8 blocks, whose render kernels
+take no notice of the staging batch and the pixels per thread: those come back
+as the defaults, and the backward's pixels per thread as what a deterministic
+plan of the tile asks for.
 The choice is cached in a JSON file keyed by GPU name, view sizes and a
 power-of-two bucket of the map size.
 
 The tile shape changes which pixels a Gaussian may reach (its 3-sigma rect is
-counted in whole tiles), so it changes the image slightly; the batch and the
-pixels per thread change only the speed.  Every tile shape is checked against
-the FP64 oracle by the test-suite.
+counted in whole tiles), so it changes the image slightly.  Every tile shape is
+checked against the FP64 oracle by the test-suite.
 """
 from __future__ import annotations
 
@@ -25,8 +25,8 @@ import torch
 from . import mapping
 
 TILES = ((8, 8), (16, 16), (32, 8))
-BATCHES = (32, 64, 128, 256)
-PPTS = (1, 2, 4, 8)
+SMEM_BATCH = 128  # the rasteriser's default
+REPEATS = 4  # timed iterations per tile, in units of `iters`
 
 
 def cache_path():
@@ -42,12 +42,16 @@ def cache_key(views, n, tight_rect=True):
     return f"{name}|{sizes}|n2^{max(0, int(math.log2(max(1, n))))}|{rects}"
 
 
-def _time_config(views, gmap, targets_packed, lam, tile, batch, ppt, iters, tight_rect=True):
+def _shape(tile):
+    return dict(smem_batch=SMEM_BATCH, pixels_per_thread=1, smem_batch_bwd=SMEM_BATCH,
+                pixels_per_thread_bwd=tile[0] * tile[1] // 32)
+
+
+def _time_tile(views, gmap, targets_packed, lam, tile, iters, tight_rect=True):
     """Mean (total, forward, backward) milliseconds of project + bin + forward +
-    loss + pixel adjoint + projection adjoint with one launch shape."""
-    rast = mapping.fit_instance_capacity(views, gmap, tile=tile, smem_batch=batch,
-                                         pixels_per_thread=ppt, smem_batch_bwd=batch,
-                                         pixels_per_thread_bwd=ppt, tight_rect=tight_rect)
+    loss + pixel adjoint + projection adjoint with one tile shape."""
+    rast = mapping.fit_instance_capacity(views, gmap, tile=tile, tight_rect=tight_rect,
+                                         **_shape(tile))
     m, g = gmap.gs_map(), gmap.gs_map_grad()
     ev = [torch.cuda.Event(enable_timing=True) for _ in range(5)]
 
@@ -99,37 +103,17 @@ def autotune(views, gmap: mapping.GaussianMap, targets_packed, lam, iters=5, use
             return dict(tile=tuple(c["tile"]), ms=c["ms"], timings=[], cached=True,
                         **{k: c[k] for k in fields})
     timings = []
-
-    def run(tile, batch, ppt):
-        t = _time_config(views, gmap, targets_packed, lam, tile, batch, ppt, iters, tight_rect)
-        timings.append(dict(tile=tile, smem_batch=batch, pixels_per_thread=ppt, ms=t[0],
+    for tile in TILES:
+        t = _time_tile(views, gmap, targets_packed, lam, tile, REPEATS * iters, tight_rect)
+        timings.append(dict(tile=tile, smem_batch=SMEM_BATCH, pixels_per_thread=1, ms=t[0],
                             fwd_ms=t[1], bwd_ms=t[2]))
         if verbose:
-            print(f"autotune {tile} batch {batch} ppt {ppt}: total {t[0]:.3f} fwd {t[1]:.3f} "
-                  f"bwd {t[2]:.3f} ms")
-
-    # stage 1: tile shape x batch at one pixel per thread, by total time
-    for tile in TILES:
-        for batch in BATCHES:
-            run(tile, batch, 1)
-    tile = min(timings, key=lambda r: r["ms"])["tile"]
-    # stage 2: pixels per thread for that tile; forward and backward launch
-    # shapes are chosen independently from their own stage times
-    for ppt in PPTS[1:]:
-        if tile[0] % ppt or (tile[0] * tile[1] // ppt) % 32:
-            continue
-        for batch in BATCHES:
-            run(tile, batch, ppt)
-    mine = [r for r in timings if r["tile"] == tile]
-    f = min(mine, key=lambda r: r["fwd_ms"])
-    b = min(mine, key=lambda r: r["bwd_ms"])
-    base = min(mine, key=lambda r: r["ms"])
-    est = base["ms"] - base["fwd_ms"] - base["bwd_ms"] + f["fwd_ms"] + b["bwd_ms"]
-    out = dict(tile=tile, smem_batch=f["smem_batch"], pixels_per_thread=f["pixels_per_thread"],
-               smem_batch_bwd=b["smem_batch"], pixels_per_thread_bwd=b["pixels_per_thread"],
-               ms=est, timings=timings, cached=False)
+            print(f"autotune {tile}: total {t[0]:.3f} fwd {t[1]:.3f} bwd {t[2]:.3f} ms")
+    best = min(timings, key=lambda r: r["ms"])
+    tile = best["tile"]
+    out = dict(tile=tile, ms=best["ms"], timings=timings, cached=False, **_shape(tile))
     if use_cache:
-        cache[key] = dict(tile=list(tile), ms=est, **{k: out[k] for k in fields})
+        cache[key] = dict(tile=list(tile), ms=out["ms"], **{k: out[k] for k in fields})
         try:
             os.makedirs(os.path.dirname(path), exist_ok=True)
             tmp = path + f".tmp{os.getpid()}"
