@@ -5,6 +5,7 @@
 #include <atomic>
 
 #include "gs_internal.cuh"
+#include "gs_occupancy.h"
 
 using namespace gs;
 
@@ -22,6 +23,20 @@ int gs::sm_count() {
         return 0;
     if (dev < kDevices && sms > 0) cache[dev].store(sms, std::memory_order_relaxed);
     return sms > 0 ? sms : 0;
+}
+
+int gs::resident_ctas(const void* kern, int threads, size_t smem) {
+    static OccupancyCache cache;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return -1;
+    return cache.get(kern, threads, smem, dev, [&] {
+        int per_sm = 0;
+        const int sms = sm_count();
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) !=
+            cudaSuccess)
+            return -1;
+        return per_sm * sms;
+    });
 }
 
 namespace {

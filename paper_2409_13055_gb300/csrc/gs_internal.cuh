@@ -148,6 +148,9 @@ inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 // and cached; 0 if the query fails.  Grid-stride kernels size their grids in
 // multiples of it.
 int sm_count();
+// CTAs of a kernel that the current device holds at once (asked once per kernel,
+// CTA size, shared memory and device), below 1 on an error.
+int resident_ctas(const void* kern, int threads, size_t smem);
 
 inline gs_status launch_status() {
     cudaError_t e = cudaGetLastError();

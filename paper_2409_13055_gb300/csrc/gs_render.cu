@@ -28,8 +28,6 @@
 //    reduce-scatter (12 shuffles, skipped when no lane touches the
 //    Gaussian), into shared memory; once per batch they become the gradient
 //    and leave as nine parallel atomics per Gaussian.
-#include <mutex>
-
 #include "gs_render.cuh"
 
 namespace gs {
@@ -991,39 +989,11 @@ static int warp_teams(int tf4) {
 }
 
 // CTAs of a persistent launch: the resident CTAs of the whole GPU, no more
-// than there are teams' worth of tiles.  The occupancy query runs once per
-// (kernel, shape, device) and is cached.
+// than there are teams' worth of tiles.
 int persistent_blocks(const void* kern, int threads, size_t smem, int tiles_per_block,
-                             int total_tiles) {
-    struct Entry {
-        const void* k;
-        int threads, dev;
-        size_t smem;
-        int blocks;
-    };
-    static Entry cache[64];
-    static int used = 0;
-    static std::mutex mu;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return -1;
-    int resident = 0;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        for (int i = 0; i < used; ++i)
-            if (cache[i].k == kern && cache[i].threads == threads && cache[i].smem == smem &&
-                cache[i].dev == dev)
-                resident = cache[i].blocks;
-        if (resident == 0) {
-            int per_sm = 0, sms = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) !=
-                    cudaSuccess ||
-                cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-                return -1;
-            resident = per_sm * sms;
-            if (resident < 1) return -1;
-            if (used < 64) cache[used++] = Entry{kern, threads, dev, smem, resident};
-        }
-    }
+                      int total_tiles) {
+    const int resident = resident_ctas(kern, threads, smem);
+    if (resident < 1) return -1;
     const int want = (total_tiles + tiles_per_block - 1) / tiles_per_block;
     return want < resident ? (want < 1 ? 1 : want) : resident;
 }

@@ -20,8 +20,6 @@
 // passes, the scan and the emission run over the visible pairs only, whose
 // count stays on the device like the instance count.  No kernel waits on
 // another block, so nothing can spin.
-#include <atomic>
-
 #include "gs_internal.cuh"
 
 namespace gs {
@@ -697,25 +695,12 @@ k_tile_order(const uint32_t* __restrict__ ranges, int T, const uint32_t* __restr
     }
 }
 
-// CTAs of a grid-stride kernel resident at once on this GPU (its occupancy
-// per SM, cached per kernel, times the SMs): the binning's kernels whose work
-// is counted on the device launch this many at most, so that no CTA is
-// launched only to find nothing to do.
+// CTAs of a grid-stride kernel resident at once on this GPU: the binning's
+// kernels whose work is counted on the device launch this many at most, so that
+// no CTA is launched only to find nothing to do.
 template <auto Kernel>
 int resident_grid(int threads, size_t smem = 0) {
-    // (a kernel's launches differ in shared memory by its digits: the last
-    // asked for is kept)
-    static std::atomic<unsigned long long> known{~0ull};
-    const unsigned long long k0 = known.load(std::memory_order_relaxed);
-    int b = (int)(k0 >> 32);
-    if (k0 == ~0ull || (k0 & 0xFFFFFFFFull) != smem) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, Kernel, threads, smem) !=
-                cudaSuccess ||
-            b < 1)
-            b = 1;
-        known.store((unsigned long long)b << 32 | smem, std::memory_order_relaxed);
-    }
-    return b * sm_count();
+    return max(sm_count(), resident_ctas(reinterpret_cast<const void*>(Kernel), threads, smem));
 }
 
 // One stable pass over up to `cap` keys (the real count comes from count_dev
