@@ -111,20 +111,13 @@ k_radix_hist(const uint32_t* __restrict__ keys, const uint32_t* count_dev, uint3
     // a grid of resident CTAs striding over the sort blocks of the active keys
     for (uint32_t blk = blockIdx.x; blk * (uint32_t)TILE < count; blk += gridDim.x) {
         const uint32_t start = blk * (uint32_t)TILE;
-        constexpr int V = ITEMS >= 4 ? ITEMS / 4 : 1;
-        constexpr uint32_t W = ITEMS >= 4 ? 4u : (uint32_t)ITEMS;  // keys per load
+        static_assert(ITEMS % 4 == 0, "whole 16-byte loads");
+        constexpr int V = ITEMS / 4;
         uint4 k[V];
 #pragma unroll
         for (int r = 0; r < V; ++r) {
-            const uint32_t i = start + W * (r * kSortThreads + threadIdx.x);
-            if (i + W <= count) {
-                if (W == 4) {
-                    k[r] = *reinterpret_cast<const uint4*>(keys + i);
-                } else {
-                    const uint2 x = *reinterpret_cast<const uint2*>(keys + i);
-                    k[r] = make_uint4(x.x, x.y, 0u, 0u);
-                }
-            }
+            const uint32_t i = start + 4u * (r * kSortThreads + threadIdx.x);
+            if (i + 4u <= count) k[r] = *reinterpret_cast<const uint4*>(keys + i);
         }
         for (int d = threadIdx.x; d <= (int)digit.mask; d += kSortThreads) h[d] = 0u;
         __syncthreads();
@@ -133,14 +126,12 @@ k_radix_hist(const uint32_t* __restrict__ keys, const uint32_t* count_dev, uint3
         };
 #pragma unroll
         for (int r = 0; r < V; ++r) {
-            const uint32_t i = start + W * (r * kSortThreads + threadIdx.x);
-            if (i + W <= count) {
+            const uint32_t i = start + 4u * (r * kSortThreads + threadIdx.x);
+            if (i + 4u <= count) {
                 add(k[r].x);
                 add(k[r].y);
-                if (W == 4) {
-                    add(k[r].z);
-                    add(k[r].w);
-                }
+                add(k[r].z);
+                add(k[r].w);
             } else {
                 for (uint32_t j = i; j < count; ++j) add(keys[j]);
             }
