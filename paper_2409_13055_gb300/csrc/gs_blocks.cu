@@ -29,10 +29,10 @@
 // 1200x680, 8x8 tiles (2.0M walked (block, Gaussian) pairs), against the kernels
 // of gs_render.cu at their best launch shape: forward 182 -> 128 us, adjoint 319 ->
 // 240 us.  Sixteen views of a 500k map: 1003 -> 629 and 1593 -> 1332 us.  200k
-// Gaussians, 640x480, 16x16 tiles: 68 -> 37 and 177 -> 74 us (there the block test
+// Gaussians, 640x480, 16x16 tiles: 68 -> 37 and 177 -> 70 us (there the block test
 // and the four warps per tile count as well).
 //
-// The sums on mma.sync (TF32, each operand in two parts) take 233 us at 1M but
+// The sums on mma.sync (TF32, each operand in two parts) take 233 us at 1M and
 // 77 at 200k, and two parts hold 22 bits of 24: every product came out low by 2e-7
 // on average, four times the rounding of the FP32 sums in the gradients of the SH
 // coefficients.  Tried and not kept: 32 slots per stage for a sixth CTA per SM (256
@@ -815,10 +815,11 @@ k_blocks_bwd(ViewTable vt, const uint32_t* __restrict__ ranges,
 // share of its SM shrinks with every other warp there, and a launch is not over
 // before its longest list, which one warp walks alone: where there are few
 // blocks, fewer warps that run faster end sooner.  Forward (8 halves),
-// at 8 / 5 / 3 / 2 CTAs per SM: 113640 blocks 632 / 696 / 897 / 1197 us, 12750
-// blocks 148 / 134 / 150 / 189, 4800 blocks 56 / 55 / 46 / 39.  Adjoint (5 halves)
-// at 5 / 3 / 2: 113640 blocks 1429 / 1798 / 2486, 12750 blocks 261 / 306 / 408, 4800
-// blocks 95 / 86 / 91.
+// at 8 / 5 / 3 / 2 CTAs per SM: 113640 blocks 628 / 673 / 823 / 1056 us, 12750
+// blocks 140 / 132 / 136 / 160, 4800 blocks 38 / 38 / 33 / 33.  Adjoint (6 halves)
+// at 5 / 3 / 2: 113640 blocks 1333 / 1591 / 2027, 12750 blocks 240 / 272 / 336, 4800
+// blocks 71 / 67 / 62; by 5 / 6 / 8 halves: 4800 blocks 65 / 61 / 61 us, 6120 blocks 87 /
+// 82 / 92, 8100 blocks 103 / 96 / 101, 4800 blocks of 16x16 tiles 75 / 70 / 70.
 int launch_ctas(const void* kern, size_t smem, int total, int per_warp2) {
     const int resident = persistent_blocks(kern, 32 * kWarps, smem, kWarps, total);
     const int sms = sm_count();
@@ -880,7 +881,7 @@ gs_status launch_blocks_bwd(const Plan* p, const uint32_t* vals, void* ws, const
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess)
         return GS_ERR_CUDA;
-    const int blocks = launch_ctas((const void*)kern, smem, total, 5);
+    const int blocks = launch_ctas((const void*)kern, smem, total, 6);
     if (blocks < 0) return GS_ERR_CUDA;
     uint32_t* queue = buf<uint32_t>(p, ws, B_TILE_QUEUE) + 1;
     if (cudaMemsetAsync(queue, 0, sizeof(uint32_t), st) != cudaSuccess) return GS_ERR_CUDA;

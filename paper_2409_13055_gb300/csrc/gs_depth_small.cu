@@ -1,6 +1,6 @@
 // gs_depth_small.cu -- the depth sort of small plans in one launch.
 //
-// The general depth sort (gs_sort.cu) is a chain of fourteen launches (three per
+// The general depth sort (gs_sort.cu) is a chain of eleven launches (three per
 // digit, two for the instance offsets); below some ten thousand pairs each of
 // them moves next to nothing and the chain's length is its time, and the host's
 // where a program launches call by call.  Here one cluster of 8 or 16 CTAs keeps the

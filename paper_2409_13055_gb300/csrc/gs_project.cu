@@ -326,7 +326,7 @@ __device__ __forceinline__ void prefetch_params(const float* __restrict__ means,
 // through; what is not finite passes too.  k_project is bound by instruction
 // issue (some 700 a pair and warp when one of its lanes is visible); with the
 // test and the row spans' halves computed once (tight_row_span): 16 views of 500k
-// 251 -> 209 us, two of 2M 195 -> 168, one of 1M 55 -> 50.  Not faster: lanes
+// 251 -> 209 us, four of 2M 195 -> 168, one of 1M 55 -> 50.  Not faster: lanes
 // walking their own views, 8 or 16 views per thread (226 and 258 us).
 struct Reach {
     float R[9], t[3];
@@ -811,10 +811,10 @@ k_project_bwd(const float* __restrict__ means, const float* __restrict__ log_sca
 // no view of the pass touches is left out altogether: its gradient is zero.  (Not
 // one whose parameters overflow or are not finite: its zeros become NaN on the
 // way, and are added.)  The groups as above.  Bound by latency at the 16 warps
-// per SM that 128 registers leave (16 views) and by the gradients' bytes (two
+// per SM that 128 registers leave (16 views) and by the gradients' bytes (four
 // views of 2M).  The colour gradients used to go through memory to a second
 // kernel for the SH sums, a thread per Gaussian reading and writing 12 of every
-// 384 bytes a plane: 16 views of 500k 285 -> 212 us, two views of 2M 287 -> 262.
+// 384 bytes a plane: 16 views of 500k 285 -> 212 us, four views of 2M 287 -> 262.
 // CTAs of 128 threads, one per 128 Gaussians: resident ones that stride end
 // unevenly (223 us).
 constexpr int kViewsThreads = 128;

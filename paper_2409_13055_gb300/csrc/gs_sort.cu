@@ -14,9 +14,9 @@
 // steps within a block (issue slots half busy, a quarter of the bandwidth), so
 // there are few of them: three over the depth, digits of up to ten bits over the
 // tile id.  Whole binning with four 8-bit depth passes and 8-bit tile digits ->
-// now: 13.8M instances of 16 views 735 -> 590 us, 3.3M of two views of 2M 280 ->
-// 260, 3.1M of one of 1M 159 -> 148, 444k of 350k pairs 65 -> 60.  The first depth pass drops the (view,
-// Gaussian) pairs the projection culled (key 0xFFFFFFFF, no tile): the later
+// now: 13.8M instances of 16 views 735 -> 590 us, 3.3M of four views of 2M 280 ->
+// 260, 3.1M of one of 1M 159 -> 148, 444k of 350k pairs 65 -> 60.  The first
+// depth pass drops the (view, Gaussian) pairs the projection culled (key 0xFFFFFFFF, no tile): the later
 // passes, the scan and the emission run over the visible pairs only, whose
 // count stays on the device like the instance count.  No kernel waits on
 // another block, so nothing can spin.
